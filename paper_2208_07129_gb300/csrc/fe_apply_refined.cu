@@ -8,8 +8,7 @@
 //   4. slave rows of Y set to 0.
 // Together Y = C^T A C X on the free rows, 0 on slave and Dirichlet rows.
 #include "fe_dispatch.cuh"
-#include "fe_evenodd.cuh"
-#include "fe_ff_body.cuh"
+#include "fe_box.cuh"
 
 namespace fe {
 
@@ -54,58 +53,18 @@ __global__ void zero_rows_kernel(T* __restrict__ Y, const int* __restrict__ rows
   }
 }
 
-template <typename T, int NP, int NQ>
-__global__ void __launch_bounds__(256) cell_apply_eo_map_kernel(const EOTables<T, NP, NQ> tab, const MeshDev m,
-                                                                const Geom<T> geo, const int* __restrict__ cells,
-                                                                int n_vec, int n_vb, const T* __restrict__ X,
-                                                                T* __restrict__ Y, const int* __restrict__ map) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  cell_body_eo<T, NP, NQ, false, false, true>(tab, m, geo, cells[blockIdx.x / n_vb], blockIdx.x % n_vb, blockDim.x,
-                                              threadIdx.x, threadIdx.y, blockDim.y, n_vec, X, Y,
-                                              reinterpret_cast<T*>(smem_raw), Scale<T>{}, map);
-}
-
-template <typename T, int NP, int NQ>
-cudaError_t launch_eo_map(const fe_ctx* c, const T* X, T* Y, int n_vec, cudaStream_t s, int want_vb,
-                          int want_lines) {
-  auto kern = cell_apply_eo_map_kernel<T, NP, NQ>;
-  const int vb = pick_vb<T, NQ>(want_vb, n_vec);
-  int nty = want_lines;
-  if (vb * nty > 256) nty = 256 / vb;
-  while ((vb * nty) % 32 != 0 && vb * nty < 256) ++nty;
-  const size_t smem = (size_t)3 * NQ * NQ * NQ * vb * sizeof(T);
-  {
-    cudaError_t e = ensure_dyn_smem(reinterpret_cast<const void*>(kern), smem);
-    if (e != cudaSuccess) return e;
-  }
-  const EOTables<T, NP, NQ> tab = make_eotables<T, NP, NQ>(c);
-  const Geom<T> geo = make_geom<T>(c);
-  const int n_vb = (n_vec + vb - 1) / vb;
-  for (int k = 0; k < c->colors.n_colors; ++k) {
-    const int n = c->colors.offset[k + 1] - c->colors.offset[k];
-    if (n == 0) continue;
-    const long long blocks = (long long)n * n_vb;
-    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    kern<<<(unsigned)blocks, dim3(vb, nty), smem, s>>>(tab, c->mdev, geo, c->d_cells + c->colors.offset[k], n_vec,
-                                                       n_vb, X, Y, c->d_map);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
 cudaError_t cells_refined(const fe_ctx* c, const void* X, void* Y, int n_vec, cudaStream_t s) {
-  const Scale<double> none{};
 #define FE_CASE(P, NQ)                                                                                       \
   if (c->p == P && c->nq == NQ) {                                                                            \
-    if (c->mode == FE_FP64)                                                                                  \
-      return launch_eo_map<double, P + 1, NQ>(c, static_cast<const double*>(X), static_cast<double*>(Y),    \
-                                              n_vec, s, c->vb64, c->nty64);                                  \
     if (c->mode == FE_FP32)                                                                                  \
-      return launch_eo_map<float, P + 1, NQ>(c, static_cast<const float*>(X), static_cast<float*>(Y), n_vec, \
-                                             s, c->vb32, c->nty32);                                          \
-    return launch_df64<P + 1, NQ, false, false, true>(c, static_cast<const double*>(X),                      \
-                                                      static_cast<double*>(Y), n_vec, s, none);              \
+      return launch_box<float, P + 1, NQ, false, true>(c, static_cast<const float*>(X), static_cast<float*>(Y), \
+                                                       n_vec, s, c->vb32, c->nty32, make_geom<float>(c));    \
+    const double* X64 = static_cast<const double*>(X);                                                       \
+    double* Y64 = static_cast<double*>(Y);                                                                   \
+    return c->mode == FE_FP64                                                                                \
+               ? launch_box<double, P + 1, NQ, false, true>(c, X64, Y64, n_vec, s, c->vb64, c->nty64,        \
+                                                            make_geom<double>(c))                            \
+               : launch_box<ff, P + 1, NQ, false, true>(c, X64, Y64, n_vec, s, c->vbdf, c->ntydf, make_geom<ff>(c)); \
   }
   FE_FOR_EACH_P_NQ(FE_CASE)
 #undef FE_CASE

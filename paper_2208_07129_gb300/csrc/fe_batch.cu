@@ -8,7 +8,7 @@
 // from the queue earlier by running CTAs, so the wait always ends (and it is
 // bounded besides: a CTA that gives up records FE_ETIMEOUT).  Within a colour
 // the cells share no node, so assembly stays conflict-free and the result is
-// bitwise the one of the per-problem launches of the even-odd line kernel
+// bitwise the one of the per-problem launches of the box-cell kernel
 // (the same cell body; Sec. 3.1.2: all cells and batches of vectors evaluated
 // concurrently, here across problems too).
 //
@@ -25,18 +25,15 @@
 #include <type_traits>
 
 #include "fe_internal.h"
-#include "fe_cell_kernel.cuh"
 #include "fe_dispatch.cuh"
-#include "fe_evenodd.cuh"
-#include "fe_ff_body.cuh"
+#include "fe_box.cuh"
 #include "../../include/fe_batch.h"
 
 namespace fe {
 
 constexpr int kBatchThreads = 128;
 constexpr int kMaxColors = 27;
-constexpr int kTabImage = 256;   // elements of an EOTables<T, NP, NQ> image (195 at p = 8, n_q = 10)
-constexpr int kKinds = 6;        // degrees 3..8 with n_q = p + 2
+constexpr int kTabImage = 256;   // elements of a BoxTables<T, NP, NQ> image (245 at p = 8, n_q = 10)
 
 template <typename T>
 struct BatchProblemDev {
@@ -44,35 +41,26 @@ struct BatchProblemDev {
   Geom<T> geo;
   int n_vec, vb, nty, kind, n_vb;
   const int* cells;                                    // colour-sorted cell ids
-  T tab[kTabImage];                                    // EOTables<T, NP, NQ> image
+  T tab[kTabImage];                                    // BoxTables<T, NP, NQ> image
 };
 
 struct WorkItem {
   int problem, color, cell_begin, cell_count, vb;
 };
 
-// Element type of X and Y for a compute type (double-float computes on FP64 data).
-template <typename T>
-struct DataOf { using type = T; };
-template <>
-struct DataOf<ff> { using type = double; };
-
 // kinds: p = 3..8 with n_q = p + 2 on affine cells
 constexpr int kind_of(int p) { return p - 3; }
 
 template <typename T, int NP, int NQ>
 __device__ __forceinline__ void run_item(const BatchProblemDev<T>& P, const WorkItem& w,
-                                         const typename DataOf<T>::type* X, typename DataOf<T>::type* Y, T* smem,
-                                         const EOTables<T, NP, NQ>& tab) {
+                                         const typename Arith<T>::D* X, typename Arith<T>::D* Y, T* smem,
+                                         const BoxTables<T, NP, NQ>& tab) {
   const int tid = threadIdx.x, vb = P.vb;
   const int v = tid % vb, ty = tid / vb, nty = kBatchThreads / vb;
   for (int c = 0; c < w.cell_count; ++c) {
     const int e = P.cells[w.cell_begin + c];
-    if constexpr (std::is_same<T, ff>::value)
-      cell_body_ff<NP, NQ, false, false>(tab, P.m, P.geo, e, w.vb, vb, v, ty, nty, P.n_vec, X, Y, smem,
-                                         Scale<double>{});
-    else
-      cell_body_eo<T, NP, NQ, false>(tab, P.m, P.geo, e, w.vb, vb, v, ty, nty, P.n_vec, X, Y, smem);
+    cell_body_box<T, NP, NQ>(tab, P.m, P.geo, e, w.vb, vb, v, ty, nty, P.n_vec, X, Y, smem,
+                             Scale<typename Arith<T>::D>{});
     __syncthreads();
   }
 }
@@ -83,14 +71,14 @@ __device__ __forceinline__ unsigned long long batch_clock_ns() {
   return t;
 }
 
-// One persistent kernel per degree (the problems of that degree, their own
-// queue): each instantiation gets the registers its cell body needs instead
-// of those of the largest degree in the batch, and the degree's 1D tables
-// (the same for all its problems) travel as a kernel parameter, so the
+// One persistent kernel per group of problems of one degree and one aspect of
+// their cells (which share the 1D tables), with its own queue: each
+// instantiation gets the registers its cell body needs instead of those of
+// the largest degree in the batch, and the group's tables travel as a kernel parameter, so the
 // contractions read their coefficients from the constant bank as in the
 // per-colour kernels.
 template <typename T, int NP, int NQ>
-__global__ void __launch_bounds__(kBatchThreads) batch_kernel(const EOTables<T, NP, NQ> tab,
+__global__ void __launch_bounds__(kBatchThreads) batch_kernel(const BoxTables<T, NP, NQ> tab,
                                                              const BatchProblemDev<T>* __restrict__ probs,
                                                              const void* const* __restrict__ ptrs,
                                                              const WorkItem* __restrict__ items, int n_items,
@@ -120,7 +108,7 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(const EOTables<T, 
       __threadfence();
     }
     __syncthreads();
-    using D = typename DataOf<T>::type;
+    using D = typename Arith<T>::D;
     const D* X = static_cast<const D*>(ptrs[2 * w.problem]);
     D* Y = static_cast<D*>(const_cast<void*>(ptrs[2 * w.problem + 1]));
     run_item<T, NP, NQ>(P, w, X, Y, smem, tab);
@@ -171,11 +159,11 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel_all(const BatchPro
     }
     for (int k = threadIdx.x; k < kTabImage; k += blockDim.x) stab[k] = P.tab[k];
     __syncthreads();
-    using D = typename DataOf<T>::type;
+    using D = typename Arith<T>::D;
     const D* X = static_cast<const D*>(ptrs[2 * w.problem]);
     D* Y = static_cast<D*>(const_cast<void*>(ptrs[2 * w.problem + 1]));
 #define FE_ITEM(K, NP, NQ) \
-  case K: run_item<T, NP, NQ>(P, w, X, Y, smem, *reinterpret_cast<const EOTables<T, NP, NQ>*>(stab)); break;
+  case K: run_item<T, NP, NQ>(P, w, X, Y, smem, *reinterpret_cast<const BoxTables<T, NP, NQ>*>(stab)); break;
     switch (P.kind) {
       FE_ITEM(0, 4, 5) FE_ITEM(1, 5, 6) FE_ITEM(2, 6, 7) FE_ITEM(3, 7, 8) FE_ITEM(4, 8, 9) FE_ITEM(5, 9, 10)
       default: break;
@@ -201,7 +189,11 @@ struct fe_batch {
   void* d_probs = nullptr;
   WorkItem* d_items = nullptr;
   int n_items = 0, n_phases = 0;
-  int item_begin[kKinds + 1] = {0};   // items of degree kind k: [item_begin[k], item_begin[k + 1])
+  // groups of problems that share one kernel and its queue: one for every
+  // problem in FP64, else one per degree and cell aspect
+  std::vector<int> group_of;           // group of each problem
+  std::vector<int> group_first;        // a problem of each group (its tables are the group's)
+  std::vector<int> item_begin;         // items of group g: [item_begin[g], item_begin[g + 1])
   int *d_next = nullptr, *d_done = nullptr, *d_need = nullptr, *d_status = nullptr;
   std::vector<int> need;               // host copy of the completion counts items wait for
   long long* d_wait_ns = nullptr;      // limit of one bounded wait (device, read by the kernels)
@@ -209,10 +201,11 @@ struct fe_batch {
   void** d_ptrs = nullptr;
   size_t smem = 0;
   int grid = 0;
-  int grid_kind[kKinds] = {0};         // persistent grid of each degree's kernel (per-degree kernels)
+  std::vector<int> group_grid;         // persistent grid of each group's kernel
   cudaStream_t cap = nullptr;
-  cudaStream_t side[kKinds] = {};       // one capture branch per degree
-  cudaEvent_t fork = nullptr, join[kKinds] = {};
+  std::vector<cudaStream_t> side;       // one capture branch per group
+  cudaEvent_t fork = nullptr;
+  std::vector<cudaEvent_t> join;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   float tune_ms = 0.f;
@@ -225,21 +218,27 @@ fe_status from_cuda(cudaError_t e) {
 }
 
 template <typename T>
-size_t tile_smem(int nq, int vb) { return (size_t)3 * nq * nq * nq * vb * sizeof(T); }
+size_t tile_smem(int nq, int vb) {
+  const int pitch[] = {0, 0, BoxTile<2>::pitch(vb), BoxTile<3>::pitch(vb), BoxTile<4>::pitch(vb), BoxTile<5>::pitch(vb),
+                       BoxTile<6>::pitch(vb), BoxTile<7>::pitch(vb), BoxTile<8>::pitch(vb), BoxTile<9>::pitch(vb),
+                       BoxTile<10>::pitch(vb)};
+  return (size_t)2 * vb * pitch[nq] * sizeof(T);
+}
 
-// The even-odd tables of one problem, copied into its table image.
+// The tables of one problem, copied into its table image.
 template <typename T, int NP, int NQ>
-void eo_image(const fe_ctx* c, T* img) {
-  static_assert(sizeof(EOTables<T, NP, NQ>) <= kTabImage * sizeof(T), "table image too small");
-  const EOTables<T, NP, NQ> t = make_eotables<T, NP, NQ>(c);
+void box_image(const fe_ctx* c, T* img) {
+  static_assert(sizeof(BoxTables<T, NP, NQ>) <= kTabImage * sizeof(T), "table image too small");
+  const BoxTables<T, NP, NQ> t = make_boxtables<T, NP, NQ>(c);
   std::memcpy(img, &t, sizeof(t));
 }
 
 // Candidate vectors-per-CTA of the autotuner for one problem.
-std::vector<int> candidates(int nq, int n_vec, size_t elem) {
+template <typename T>
+std::vector<int> candidates(int nq, int n_vec) {
   std::vector<int> out;
   for (int vb : {2, 4, 8, 16, 32}) {
-    if ((size_t)3 * nq * nq * nq * vb * elem > 110 * 1024) continue;   // keep two CTAs per SM
+    if (tile_smem<T>(nq, vb) > 110 * 1024) continue;   // keep two CTAs per SM
     if (vb > 1 && vb / 2 >= n_vec) continue;
     out.push_back(vb);
   }
@@ -252,9 +251,10 @@ std::vector<int> candidates(int nq, int n_vec, size_t elem) {
 // narrowest tile for its parallelism alone) with the problem's degree and
 // block width (capped at 64 vectors) for every candidate tile; return the
 // fastest vectors-per-CTA.
+template <typename T>
 int autotune(const fe_ctx* c, int n_vec_full, fe_mode mode, float* spent_ms) {
   const size_t elem = mode == FE_FP32 ? 4 : 8;
-  std::vector<int> cand = candidates(c->nq, n_vec_full, elem);
+  std::vector<int> cand = candidates<T>(c->nq, n_vec_full);
   if (cand.size() == 1) return cand[0];
   const int n_vec = std::min(n_vec_full, 64);
   fe_mesh_desc md{};
@@ -275,7 +275,7 @@ int autotune(const fe_ctx* c, int n_vec_full, fe_mode mode, float* spent_ms) {
     cudaEventCreate(&b);
     float best_ms = 1e30f;
     for (int vb : cand) {
-      fe_set_tile(px, mode, vb, kBatchThreads / vb, mode == FE_FP32 ? 3 : 0);   // the even-odd line kernel
+      fe_set_tile(px, mode, vb, kBatchThreads / vb, mode == FE_FP32 ? 3 : 0);   // the box-cell kernel
       fe_apply(px, X, Y, n_vec, nullptr);
       cudaEventRecord(a);
       for (int r = 0; r < 3; ++r) fe_apply(px, X, Y, n_vec, nullptr);
@@ -296,11 +296,11 @@ int autotune(const fe_ctx* c, int n_vec_full, fe_mode mode, float* spent_ms) {
   return best;
 }
 
-// The persistent kernel of one degree: before the capture, its shared-memory
+// The persistent kernel of one group: before the capture, its shared-memory
 // attribute and its grid = occupancy x SMs (at most one CTA per work item);
 // then its launch, recorded into the graph.
 template <typename T, int NP, int NQ>
-cudaError_t prepare_kind(fe_batch* b, int kind, int n_k, size_t smem) {
+cudaError_t prepare_group(fe_batch* b, int g, int n_g, size_t smem) {
   auto kern = batch_kernel<T, NP, NQ>;
   cudaError_t e = ensure_dyn_smem(reinterpret_cast<const void*>(kern), smem);
   int per_sm = 0, sms = 0, dev = 0;
@@ -308,37 +308,41 @@ cudaError_t prepare_kind(fe_batch* b, int kind, int n_k, size_t smem) {
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  b->grid_kind[kind] = std::max(1, std::min(n_k, std::max(1, per_sm) * sms));
-  b->grid = std::max(b->grid, b->grid_kind[kind]);
+  b->group_grid[g] = std::max(1, std::min(n_g, std::max(1, per_sm) * sms));
+  b->grid = std::max(b->grid, b->group_grid[g]);
   return cudaSuccess;
 }
 
 template <typename T, int NP, int NQ>
-cudaError_t launch_kind(fe_batch* b, int kind, int n_k, size_t smem) {
+cudaError_t launch_group(fe_batch* b, int g, int n_g, size_t smem) {
   auto kern = batch_kernel<T, NP, NQ>;
-  const fe_ctx* c0 = nullptr;   // the degree's tables: those of its first problem (all equal)
-  for (int i = 0; i < b->n && !c0; ++i)
-    if (kind_of(b->ctxs[i]->p) == kind) c0 = b->ctxs[i];
-  if (!c0) return cudaErrorInvalidValue;
-  const EOTables<T, NP, NQ> tab = make_eotables<T, NP, NQ>(c0);
-  kern<<<b->grid_kind[kind], kBatchThreads, smem, b->side[kind]>>>(
+  const BoxTables<T, NP, NQ> tab = make_boxtables<T, NP, NQ>(b->ctxs[b->group_first[g]]);
+  kern<<<b->group_grid[g], kBatchThreads, smem, b->side[g]>>>(
       tab, static_cast<const BatchProblemDev<T>*>(b->d_probs), const_cast<const void* const*>(b->d_ptrs),
-      b->d_items + b->item_begin[kind], n_k, b->d_next + kind, b->d_done, b->d_need, b->d_status, b->d_wait_ns);
+      b->d_items + b->item_begin[g], n_g, b->d_next + g, b->d_done, b->d_need, b->d_status, b->d_wait_ns);
   return cudaGetLastError();
 }
 
-// Both steps for kind k (p = k + 3, n_q = p + 2).
+// Both steps for group g (degree p, n_q = p + 2).
 template <typename T>
-cudaError_t for_kind(fe_batch* b, int kind, int n_k, size_t smem, bool launch) {
-  switch (kind) {
-    case 0: return launch ? launch_kind<T, 4, 5>(b, kind, n_k, smem) : prepare_kind<T, 4, 5>(b, kind, n_k, smem);
-    case 1: return launch ? launch_kind<T, 5, 6>(b, kind, n_k, smem) : prepare_kind<T, 5, 6>(b, kind, n_k, smem);
-    case 2: return launch ? launch_kind<T, 6, 7>(b, kind, n_k, smem) : prepare_kind<T, 6, 7>(b, kind, n_k, smem);
-    case 3: return launch ? launch_kind<T, 7, 8>(b, kind, n_k, smem) : prepare_kind<T, 7, 8>(b, kind, n_k, smem);
-    case 4: return launch ? launch_kind<T, 8, 9>(b, kind, n_k, smem) : prepare_kind<T, 8, 9>(b, kind, n_k, smem);
-    case 5: return launch ? launch_kind<T, 9, 10>(b, kind, n_k, smem) : prepare_kind<T, 9, 10>(b, kind, n_k, smem);
+cudaError_t for_group(fe_batch* b, int g, size_t smem, bool launch) {
+  const int n_g = b->item_begin[g + 1] - b->item_begin[g];
+  switch (kind_of(b->ctxs[b->group_first[g]]->p)) {
+    case 0: return launch ? launch_group<T, 4, 5>(b, g, n_g, smem) : prepare_group<T, 4, 5>(b, g, n_g, smem);
+    case 1: return launch ? launch_group<T, 5, 6>(b, g, n_g, smem) : prepare_group<T, 5, 6>(b, g, n_g, smem);
+    case 2: return launch ? launch_group<T, 6, 7>(b, g, n_g, smem) : prepare_group<T, 6, 7>(b, g, n_g, smem);
+    case 3: return launch ? launch_group<T, 7, 8>(b, g, n_g, smem) : prepare_group<T, 7, 8>(b, g, n_g, smem);
+    case 4: return launch ? launch_group<T, 8, 9>(b, g, n_g, smem) : prepare_group<T, 8, 9>(b, g, n_g, smem);
+    case 5: return launch ? launch_group<T, 9, 10>(b, g, n_g, smem) : prepare_group<T, 9, 10>(b, g, n_g, smem);
     default: return cudaErrorInvalidValue;
   }
+}
+
+// Whether two problems share their 1D tables: the degree (and so n_q) and the
+// cells' aspect (the stiffness tables carry its ratios).
+bool same_tables(const fe_ctx* a, const fe_ctx* b) {
+  return a->p == b->p && a->box_h[2] / a->box_h[0] == b->box_h[2] / b->box_h[0] &&
+         a->box_h[2] / a->box_h[1] == b->box_h[2] / b->box_h[1];
 }
 
 template <typename T>
@@ -364,12 +368,12 @@ fe_status build_batch(fe_batch* b, int autotune_on) {
     int vb;
     auto key = std::make_pair(c->p, bucket);
     if (!autotune_on) {
-      vb = candidates(c->nq, P.n_vec, sizeof(T)).back();
+      vb = candidates<T>(c->nq, P.n_vec).back();
       vb = std::min(vb, 8);
     } else if (tuned.count(key)) {
       vb = tuned[key];
     } else {
-      vb = autotune(c, P.n_vec, b->mode, &b->tune_ms);
+      vb = autotune<T>(c, P.n_vec, b->mode, &b->tune_ms);
       tuned[key] = vb;
     }
     P.vb = vb;
@@ -378,28 +382,41 @@ fe_status build_batch(fe_batch* b, int autotune_on) {
     b->vb[i] = vb;
     std::memset(P.tab, 0, sizeof(P.tab));
     switch (P.kind) {
-      case 0: eo_image<T, 4, 5>(c, P.tab); break;
-      case 1: eo_image<T, 5, 6>(c, P.tab); break;
-      case 2: eo_image<T, 6, 7>(c, P.tab); break;
-      case 3: eo_image<T, 7, 8>(c, P.tab); break;
-      case 4: eo_image<T, 8, 9>(c, P.tab); break;
-      case 5: eo_image<T, 9, 10>(c, P.tab); break;
+      case 0: box_image<T, 4, 5>(c, P.tab); break;
+      case 1: box_image<T, 5, 6>(c, P.tab); break;
+      case 2: box_image<T, 6, 7>(c, P.tab); break;
+      case 3: box_image<T, 7, 8>(c, P.tab); break;
+      case 4: box_image<T, 8, 9>(c, P.tab); break;
+      case 5: box_image<T, 9, 10>(c, P.tab); break;
       default: break;
     }
     smem = std::max(smem, tile_smem<T>(c->nq, vb));
   }
-  // work items, phase-major: one queue over all problems (FP64, merged
-  // kernel) or one queue per degree (per-degree kernels)
+  // groups: every problem (FP64, merged kernel), or the problems that share
+  // their tables (one kernel and one queue each)
   constexpr bool merged = std::is_same<T, double>::value;
+  b->group_of.assign(n, 0);
+  for (int i = 0; i < n; ++i) {
+    int g = 0;
+    const int ng = (int)b->group_first.size();
+    while (g < ng && !merged && !same_tables(b->ctxs[b->group_first[g]], b->ctxs[i])) ++g;
+    if (g == ng) b->group_first.push_back(i);
+    b->group_of[i] = g;
+  }
+  const int groups = (int)b->group_first.size();
+  b->group_grid.assign(groups, 0);
+  b->side.assign(groups, nullptr);
+  b->join.assign(groups, nullptr);
+  // work items, phase-major within each group
   std::vector<WorkItem> items;
   int phases = 0;
-  for (int kind = 0; kind < (merged ? 1 : kKinds); ++kind) {
-  b->item_begin[kind] = (int)items.size();
+  for (int g = 0; g < groups; ++g) {
+  b->item_begin.push_back((int)items.size());
   for (int k = 0; k < kMaxColors; ++k) {
     bool any = false;
     for (int i = 0; i < n; ++i) {
       fe_ctx* c = b->ctxs[i];
-      if ((!merged && hp[i].kind != kind) || k >= c->colors.n_colors) continue;
+      if (b->group_of[i] != g || k >= c->colors.n_colors) continue;
       any = true;
       const int c0 = c->colors.offset[k], c1 = c->colors.offset[k + 1];
       const BatchProblemDev<T>& P = hp[i];
@@ -417,7 +434,7 @@ fe_status build_batch(fe_batch* b, int autotune_on) {
     if (any) phases = std::max(phases, k + 1);
   }
   }
-  for (int kind = merged ? 1 : kKinds; kind <= kKinds; ++kind) b->item_begin[kind] = (int)items.size();
+  b->item_begin.push_back((int)items.size());
   b->n_items = (int)items.size();
   b->n_phases = phases;
   b->smem = smem;
@@ -430,7 +447,7 @@ fe_status build_batch(fe_batch* b, int autotune_on) {
   if (e == cudaSuccess) e = cudaMalloc(&b->d_need, need.size() * sizeof(int));
   if (e == cudaSuccess) e = cudaMemcpy(b->d_need, need.data(), need.size() * sizeof(int), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMalloc(&b->d_done, need.size() * sizeof(int));
-  if (e == cudaSuccess) e = cudaMalloc(&b->d_next, kKinds * sizeof(int));
+  if (e == cudaSuccess) e = cudaMalloc(&b->d_next, groups * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&b->d_status, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(b->d_status, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&b->d_wait_ns, sizeof(long long));
@@ -443,8 +460,8 @@ fe_status build_batch(fe_batch* b, int autotune_on) {
   if (e == cudaSuccess) e = cudaMallocHost(&b->h_ptrs, 2 * n * sizeof(void*));
   if (e != cudaSuccess) return fe::cuda_status(e, where);
   // graph: reset the queues and the colour counters, then one persistent
-  // kernel per degree present, as parallel branches (the degrees share the
-  // GPU, and one degree's tail overlaps the others' work).  Every wait of a
+  // kernel per group, as parallel branches (the groups share the GPU, and one
+  // group's tail overlaps the others' work).  Every wait of a
   // CTA is on items its own kernel dequeued earlier, whose CTAs are running,
   // so concurrent branches cannot block each other.
   // kernel attributes and grids first: the capture below only records work
@@ -458,21 +475,18 @@ fe_status build_batch(fe_batch* b, int autotune_on) {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     b->grid = std::max(1, std::min(b->n_items, std::max(1, per_sm) * sms));
   } else {
-    for (int kind = 0; kind < kKinds && e == cudaSuccess; ++kind) {
-      const int n_k = b->item_begin[kind + 1] - b->item_begin[kind];
-      if (n_k > 0) e = for_kind<T>(b, kind, n_k, smem, false);
-    }
+    for (int g = 0; g < groups && e == cudaSuccess; ++g) e = for_group<T>(b, g, smem, false);
   }
   if (e != cudaSuccess) return fe::cuda_status(e, where);
   where = "fe_batch_create: streams and events";
   e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
-  for (int k = 0; k < kKinds && e == cudaSuccess; ++k) e = cudaStreamCreateWithFlags(&b->side[k], cudaStreamNonBlocking);
+  for (int k = 0; k < groups && e == cudaSuccess; ++k) e = cudaStreamCreateWithFlags(&b->side[k], cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
-  for (int k = 0; k < kKinds && e == cudaSuccess; ++k) e = cudaEventCreateWithFlags(&b->join[k], cudaEventDisableTiming);
+  for (int k = 0; k < groups && e == cudaSuccess; ++k) e = cudaEventCreateWithFlags(&b->join[k], cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
   if (e == cudaSuccess) {
     where = "fe_batch_create: captured launches";
-    cudaMemsetAsync(b->d_next, 0, kKinds * sizeof(int), b->cap);
+    cudaMemsetAsync(b->d_next, 0, groups * sizeof(int), b->cap);
     cudaMemsetAsync(b->d_done, 0, need.size() * sizeof(int), b->cap);
     cudaEventRecord(b->fork, b->cap);
     if constexpr (merged) {
@@ -485,16 +499,14 @@ fe_status build_batch(fe_batch* b, int autotune_on) {
       e = cudaGetLastError();
       if (e != cudaSuccess) where = "fe_batch_create: captured resets of the queues";
     }
-    for (int kind = 0; kind < kKinds && e == cudaSuccess && !merged; ++kind) {
-      const int n_k = b->item_begin[kind + 1] - b->item_begin[kind];
-      if (n_k == 0) continue;
-      e = cudaStreamWaitEvent(b->side[kind], b->fork, 0);
-      if (e != cudaSuccess) { where = "fe_batch_create: fork of a degree's branch"; break; }
-      e = for_kind<T>(b, kind, n_k, smem, true);
-      if (e != cudaSuccess) { where = "fe_batch_create: captured launch of a degree's kernel"; break; }
-      e = cudaEventRecord(b->join[kind], b->side[kind]);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(b->cap, b->join[kind], 0);
-      if (e != cudaSuccess) where = "fe_batch_create: join of a degree's branch";
+    for (int g = 0; g < groups && e == cudaSuccess && !merged; ++g) {
+      e = cudaStreamWaitEvent(b->side[g], b->fork, 0);
+      if (e != cudaSuccess) { where = "fe_batch_create: fork of a group's branch"; break; }
+      e = for_group<T>(b, g, smem, true);
+      if (e != cudaSuccess) { where = "fe_batch_create: captured launch of a group's kernel"; break; }
+      e = cudaEventRecord(b->join[g], b->side[g]);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(b->cap, b->join[g], 0);
+      if (e != cudaSuccess) where = "fe_batch_create: join of a group's branch";
     }
     cudaGraph_t g = nullptr;
     const cudaError_t e2 = cudaStreamEndCapture(b->cap, &g);
@@ -597,10 +609,10 @@ extern "C" void fe_batch_destroy(fe_batch* b) {
   if (b->exec) cudaGraphExecDestroy(b->exec);
   if (b->graph) cudaGraphDestroy(b->graph);
   if (b->cap) cudaStreamDestroy(b->cap);
-  for (int k = 0; k < kKinds; ++k) {
-    if (b->side[k]) cudaStreamDestroy(b->side[k]);
-    if (b->join[k]) cudaEventDestroy(b->join[k]);
-  }
+  for (cudaStream_t st : b->side)
+    if (st) cudaStreamDestroy(st);
+  for (cudaEvent_t ev : b->join)
+    if (ev) cudaEventDestroy(ev);
   if (b->fork) cudaEventDestroy(b->fork);
   cudaFree(b->d_probs); cudaFree(b->d_items); cudaFree(b->d_need); cudaFree(b->d_done); cudaFree(b->d_next);
   cudaFree(b->d_status); cudaFree(b->d_ptrs); cudaFree(b->d_wait_ns);

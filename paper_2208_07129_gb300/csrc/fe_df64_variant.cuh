@@ -4,6 +4,7 @@
 // of each compile in parallel with the others.
 #pragma once
 
+#include "fe_box.cuh"
 #include "fe_ff_body.cuh"
 
 namespace fe {
@@ -12,7 +13,10 @@ template <bool GEN, bool SC>
 cudaError_t apply_df64_variant(const fe_ctx* c, const double* X, double* Y, int n_vec, cudaStream_t s,
                                const Scale<double>& sc) {
 #define FE_CASE(P, NQ) \
-  if (c->p == P && c->nq == NQ) return launch_df64<P + 1, NQ, GEN, SC>(c, X, Y, n_vec, s, sc);
+  if (c->p == P && c->nq == NQ) {                                                                     \
+    if constexpr (GEN) return launch_df64<P + 1, NQ, SC>(c, X, Y, n_vec, s, sc);                       \
+    else return launch_box<ff, P + 1, NQ, SC>(c, X, Y, n_vec, s, c->vbdf, c->ntydf, make_geom<ff>(c), sc); \
+  }
   FE_FOR_EACH_P_NQ(FE_CASE)
 #undef FE_CASE
   return cudaErrorInvalidValue;

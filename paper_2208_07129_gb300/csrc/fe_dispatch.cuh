@@ -28,6 +28,10 @@ template <>
 inline Geom<float> make_geom<float>(const fe_ctx* c) {
   return Geom<float>{c->d_cellG32, c->d_ptG32, c->d_ptC32};
 }
+template <>
+inline Geom<ff> make_geom<ff>(const fe_ctx* c) {
+  return Geom<ff>{c->d_cellGff, c->d_ptGff, c->d_ptCff};
+}
 
 // Vectors per CTA: the largest power of two not above `want`, the padded
 // n_vec, and what three n_q^3 x B tiles allow in 200 KB of shared memory.

@@ -17,7 +17,7 @@
 
 #include <algorithm>
 
-#include "fe_cell_kernel.cuh"
+#include "fe_dispatch.cuh"
 
 namespace fe {
 
@@ -61,18 +61,17 @@ __device__ __forceinline__ void eo_apply(const EOTab<T, NO, NI>& t, const T* in,
   }
 }
 
-// Same as cell_body (identical data flow, tiles and assembly, the same SC
-// epilogue), with every 1D contraction in even-odd form.  With MAP the cell's
-// nodes come from an explicit map (see map_node) instead of the structured
-// numbering: the refined meshes with hanging nodes.
+// Trilinear cells: same as cell_body (identical data flow, tiles and assembly,
+// the same SC epilogue), with every 1D contraction in even-odd form.  Box
+// cells run the kernel of fe_box.cuh.
 // LOCAL: the cell's result is written to Y[(e n_p^3 + local node) n_vec + v]
 // (a per-cell scratch block, every local node, constrained ones included)
 // instead of being assembled into the global vector.
-template <typename T, int NP, int NQ, bool GEN, bool SC = false, bool MAP = false, bool LOCAL = false>
+template <typename T, int NP, int NQ, bool SC = false, bool LOCAL = false>
 __device__ __forceinline__ void cell_body_eo(const EOTables<T, NP, NQ>& tab, const MeshDev& m, const Geom<T>& geo,
                                              int e, int vb, int B, int v, int ty, int nty, int n_vec,
                                              const T* __restrict__ X, T* __restrict__ Y, T* smem,
-                                             const Scale<T>& sc = Scale<T>{}, const int* __restrict__ map = nullptr) {
+                                             const Scale<T>& sc = Scale<T>{}) {
   constexpr int P = NP - 1;
   constexpr int NQ3 = NQ * NQ * NQ;
   T* ST = smem;
@@ -91,17 +90,9 @@ __device__ __forceinline__ void cell_body_eo(const EOTables<T, NP, NQ>& tab, con
     T u[NP], a[NQ];
 #pragma unroll
     for (int i1 = 0; i1 < NP; ++i1) {
-      size_t node;
-      bool con;
-      if constexpr (MAP) {
-        const int code = __ldg(map + (size_t)e * NP * NP * NP + l * NP + i1);
-        node = (size_t)(code & kMapIndex);
-        con = (code & kMapConstrained) != 0;
-      } else {
-        const int gx = node_coord(cx, i1, P, m.Nx, m.periodic);
-        node = row + gx;
-        con = con_yz || on_boundary(gx, m.Nx, m.periodic);
-      }
+      const int gx = node_coord(cx, i1, P, m.Nx, m.periodic);
+      const size_t node = row + gx;
+      const bool con = con_yz || on_boundary(gx, m.Nx, m.periodic);
       u[i1] = (active && !con) ? __ldg(X + node * n_vec + vg) : T(0);
       if constexpr (SC) u[i1] *= __ldg(sc.msq + node);
     }
@@ -147,13 +138,6 @@ __device__ __forceinline__ void cell_body_eo(const EOTables<T, NP, NQ>& tab, con
   }
   __syncthreads();
   // ---- z-lines: gradient along z, quadrature-point operation, transposed z pass ----
-  // Cells without per-point geometry are axis-aligned boxes (checked at
-  // setup): their metric is diagonal, and the point operation scales each
-  // gradient component by one coefficient.
-  T g00, g01, g02, g11, g12, g22;
-  if (!GEN) {
-    g00 = geo.cellG[e * 6 + 0]; g11 = geo.cellG[e * 6 + 3]; g22 = geo.cellG[e * 6 + 5];
-  }
   const T* ptC = geo.ptC + (size_t)e * NQ3;
   for (int l = ty; l < NQ * NQ; l += nty) {
     T t[NQ], h2[NQ], o[NQ];
@@ -165,17 +149,11 @@ __device__ __forceinline__ void cell_body_eo(const EOTables<T, NP, NQ>& tab, con
       const T d2 = h2[q];
       const int Q = q * NQ * NQ + l;
       const T d0 = S0[Q * B + v], d1 = S1[Q * B + v];
-      if (GEN) {
-        const T* pg = geo.ptG + (size_t)e * 6 * NQ3 + Q;
-        g00 = pg[0]; g01 = pg[NQ3]; g02 = pg[2 * NQ3]; g11 = pg[3 * NQ3]; g12 = pg[4 * NQ3]; g22 = pg[5 * NQ3];
-        S0[Q * B + v] = g00 * d0 + g01 * d1 + g02 * d2;
-        S1[Q * B + v] = g01 * d0 + g11 * d1 + g12 * d2;
-        h2[q] = g02 * d0 + g12 * d1 + g22 * d2;
-      } else {
-        S0[Q * B + v] = g00 * d0;
-        S1[Q * B + v] = g11 * d1;
-        h2[q] = g22 * d2;
-      }
+      const T* pg = geo.ptG + (size_t)e * 6 * NQ3 + Q;
+      const T g00 = pg[0], g01 = pg[NQ3], g02 = pg[2 * NQ3], g11 = pg[3 * NQ3], g12 = pg[4 * NQ3], g22 = pg[5 * NQ3];
+      S0[Q * B + v] = g00 * d0 + g01 * d1 + g02 * d2;
+      S1[Q * B + v] = g01 * d0 + g11 * d1 + g12 * d2;
+      h2[q] = g02 * d0 + g12 * d1 + g22 * d2;
       t[q] = ptC[Q] * t[q];
     }
     eo_apply<T, NQ, NQ, -1>(tab.Dt, h2, o);
@@ -247,19 +225,10 @@ __device__ __forceinline__ void cell_body_eo(const EOTables<T, NP, NQ>& tab, con
     const size_t row = (size_t)(gy + (size_t)m.Ny * gz) * m.Nx;
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
-      size_t node;
-      bool con, first;
-      if constexpr (MAP) {
-        const int code = __ldg(map + (size_t)e * NP * NP * NP + l * NP + i);
-        node = (size_t)(code & kMapIndex);
-        con = (code & kMapConstrained) != 0;
-        first = (code & kMapFirst) != 0;
-      } else {
-        const int gx = node_coord(cx, i, P, m.Nx, m.periodic);
-        node = row + gx;
-        con = con_yz || on_boundary(gx, m.Nx, m.periodic);
-        first = first_yz && first_along(cx, m.nx, i, P, m.periodic, m.last_odd_x);
-      }
+      const int gx = node_coord(cx, i, P, m.Nx, m.periodic);
+      const size_t node = row + gx;
+      const bool con = con_yz || on_boundary(gx, m.Nx, m.periodic);
+      const bool first = first_yz && first_along(cx, m.nx, i, P, m.periodic, m.last_odd_x);
       T* dst = Y + node * n_vec + vg;
       if constexpr (SC) {
         scaled_store(dst, X + node * n_vec + vg, sc.a * __ldg(sc.msq + node) * o[i], first, con, sc);
@@ -271,35 +240,35 @@ __device__ __forceinline__ void cell_body_eo(const EOTables<T, NP, NQ>& tab, con
   }
 }
 
-template <typename T, int NP, int NQ, bool GEN>
+template <typename T, int NP, int NQ>
 __global__ void __launch_bounds__(256) cell_apply_eo_kernel(const EOTables<T, NP, NQ> tab, const MeshDev m,
                                                             const Geom<T> geo, const int* __restrict__ cells,
                                                             int n_vec, int n_vb, const T* __restrict__ X,
                                                             T* __restrict__ Y) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cell_body_eo<T, NP, NQ, GEN>(tab, m, geo, cells[blockIdx.x / n_vb], blockIdx.x % n_vb, blockDim.x, threadIdx.x,
+  cell_body_eo<T, NP, NQ>(tab, m, geo, cells[blockIdx.x / n_vb], blockIdx.x % n_vb, blockDim.x, threadIdx.x,
                                threadIdx.y, blockDim.y, n_vec, X, Y, reinterpret_cast<T*>(smem_raw));
 }
 
 // The scaled product of the Chebyshev filter with even-odd contractions.
-template <typename T, int NP, int NQ, bool GEN>
+template <typename T, int NP, int NQ>
 __global__ void __launch_bounds__(256) cell_apply_eo_scaled_kernel(const EOTables<T, NP, NQ> tab, const MeshDev m,
                                                                    const Geom<T> geo, const int* __restrict__ cells,
                                                                    int n_vec, int n_vb, const T* __restrict__ X,
                                                                    T* __restrict__ Y, const Scale<T> sc) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cell_body_eo<T, NP, NQ, GEN, true>(tab, m, geo, cells[blockIdx.x / n_vb], blockIdx.x % n_vb, blockDim.x,
+  cell_body_eo<T, NP, NQ, true>(tab, m, geo, cells[blockIdx.x / n_vb], blockIdx.x % n_vb, blockDim.x,
                                      threadIdx.x, threadIdx.y, blockDim.y, n_vec, X, Y,
                                      reinterpret_cast<T*>(smem_raw), sc);
 }
 
 // Small meshes: every cell in one launch, results to the per-cell scratch W.
-template <typename T, int NP, int NQ, bool GEN>
+template <typename T, int NP, int NQ>
 __global__ void __launch_bounds__(256) cell_apply_eo_local_kernel(const EOTables<T, NP, NQ> tab, const MeshDev m,
                                                                   const Geom<T> geo, int n_vec, int n_vb,
                                                                   const T* __restrict__ X, T* __restrict__ W) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cell_body_eo<T, NP, NQ, GEN, false, false, true>(tab, m, geo, blockIdx.x / n_vb, blockIdx.x % n_vb, blockDim.x,
+  cell_body_eo<T, NP, NQ, false, true>(tab, m, geo, blockIdx.x / n_vb, blockIdx.x % n_vb, blockDim.x,
                                                    threadIdx.x, threadIdx.y, blockDim.y, n_vec, X, W,
                                                    reinterpret_cast<T*>(smem_raw));
 }
@@ -392,12 +361,12 @@ EOTables<T, NP, NQ> make_eotables(const fe_ctx* c) {
   return t;
 }
 
-template <typename T, int NP, int NQ, bool GEN, bool SC = false>
+template <typename T, int NP, int NQ, bool SC = false>
 cudaError_t launch_apply_eo(const fe_ctx* c, const T* X, T* Y, int n_vec, cudaStream_t s, int want_vb,
                             int want_lines, const Scale<T>& sc = Scale<T>{}) {
   const void* kern;
-  if constexpr (SC) kern = reinterpret_cast<const void*>(cell_apply_eo_scaled_kernel<T, NP, NQ, GEN>);
-  else kern = reinterpret_cast<const void*>(cell_apply_eo_kernel<T, NP, NQ, GEN>);
+  if constexpr (SC) kern = reinterpret_cast<const void*>(cell_apply_eo_scaled_kernel<T, NP, NQ>);
+  else kern = reinterpret_cast<const void*>(cell_apply_eo_kernel<T, NP, NQ>);
   const int vb = pick_vb<T, NQ>(want_vb, n_vec);
   int nty = want_lines;
   if (vb * nty > 256) nty = 256 / vb;
@@ -414,7 +383,7 @@ cudaError_t launch_apply_eo(const fe_ctx* c, const T* X, T* Y, int n_vec, cudaSt
     // (one vector per CTA, so even a few cells fill the GPU) writing each
     // cell's result to the scratch, then one gather in colour order.
     if (c->d_small && (size_t)n_vec * NP * NP * NP * c->n_cells * sizeof(T) <= c->small_bytes) {
-      auto lk = cell_apply_eo_local_kernel<T, NP, NQ, GEN>;
+      auto lk = cell_apply_eo_local_kernel<T, NP, NQ>;
       constexpr int lines = NQ * NQ < 64 ? 32 : 64;
       const size_t lsm = (size_t)3 * NQ * NQ * NQ * sizeof(T);
       cudaError_t e = ensure_dyn_smem(reinterpret_cast<const void*>(lk), lsm);
@@ -435,10 +404,10 @@ cudaError_t launch_apply_eo(const fe_ctx* c, const T* X, T* Y, int n_vec, cudaSt
     const long long blocks = (long long)n * n_vb;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     if constexpr (SC)
-      cell_apply_eo_scaled_kernel<T, NP, NQ, GEN><<<(unsigned)blocks, dim3(vb, nty), smem, s>>>(
+      cell_apply_eo_scaled_kernel<T, NP, NQ><<<(unsigned)blocks, dim3(vb, nty), smem, s>>>(
           tab, c->mdev, geo, c->d_cells + c->colors.offset[k], n_vec, n_vb, X, Y, sc);
     else
-      cell_apply_eo_kernel<T, NP, NQ, GEN><<<(unsigned)blocks, dim3(vb, nty), smem, s>>>(
+      cell_apply_eo_kernel<T, NP, NQ><<<(unsigned)blocks, dim3(vb, nty), smem, s>>>(
           tab, c->mdev, geo, c->d_cells + c->colors.offset[k], n_vec, n_vb, X, Y);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;

@@ -1,6 +1,6 @@
 // FE_DF64: FP64 data, the cell body in double-float arithmetic (fe_ff.cuh).
 //
-// Same data flow, tiles, tables and colour-ordered assembly as the FP64
+// Trilinear cells (box cells: fe_box.cuh with Arith<ff>).  Same data flow, tiles, tables and colour-ordered assembly as the FP64
 // even-odd line kernel (fe_evenodd.cuh); only the arithmetic differs.  Every
 // 1D contraction output is one compensated dot product (acc_first /
 // acc_fma / acc_value), the even/odd pre- and post-combinations are
@@ -9,7 +9,7 @@
 // added back to FP64 on the scatter, and the colour-ordered accumulation of
 // Y stays in FP64.  Error: about 2^-44 relative per contraction, ~1e-14 on
 // the product (against 1e-12 allowed for FP64).  Instantiated in
-// fe_df64.cu (structured meshes) and fe_apply_refined.cu (explicit maps).
+// fe_df64_general.cu and fe_df64_scaled_general.cu.
 #pragma once
 
 #include "fe_dispatch.cuh"
@@ -50,11 +50,11 @@ __device__ __forceinline__ void eo_apply_ff(const EOTab<ff, NO, NI>& t, const ff
 // SC: the scaled product of the Chebyshev filter (see Scale); the M^-1/2
 // scalings and the b X + c Y terms are applied in FP64 at the gather and the
 // scatter.
-template <int NP, int NQ, bool GEN, bool SC, bool MAP = false>
+template <int NP, int NQ, bool SC>
 __device__ __forceinline__ void cell_body_ff(const EOTables<ff, NP, NQ>& tab, const MeshDev& m, const Geom<ff>& geo,
                                              int e, int vb, int B, int v, int ty, int nty, int n_vec,
                                              const double* __restrict__ X, double* __restrict__ Y, ff* smem,
-                                             const Scale<double>& sc, const int* __restrict__ map = nullptr) {
+                                             const Scale<double>& sc) {
   constexpr int P = NP - 1;
   constexpr int NQ3 = NQ * NQ * NQ;
   ff* ST = smem;
@@ -73,17 +73,9 @@ __device__ __forceinline__ void cell_body_ff(const EOTables<ff, NP, NQ>& tab, co
     ff u[NP], a[NQ];
 #pragma unroll
     for (int i1 = 0; i1 < NP; ++i1) {
-      size_t node;
-      bool con;
-      if constexpr (MAP) {
-        const int code = __ldg(map + (size_t)e * NP * NP * NP + l * NP + i1);
-        node = (size_t)(code & kMapIndex);
-        con = (code & kMapConstrained) != 0;
-      } else {
-        const int gx = node_coord(cx, i1, P, m.Nx, m.periodic);
-        node = row + gx;
-        con = con_yz || on_boundary(gx, m.Nx, m.periodic);
-      }
+      const int gx = node_coord(cx, i1, P, m.Nx, m.periodic);
+      const size_t node = row + gx;
+      const bool con = con_yz || on_boundary(gx, m.Nx, m.periodic);
       double x = (active && !con) ? __ldg(X + node * n_vec + vg) : 0.0;
       if constexpr (SC) x *= __ldg(sc.msq + node);
       u[i1] = ff(x);
@@ -130,11 +122,6 @@ __device__ __forceinline__ void cell_body_ff(const EOTables<ff, NP, NQ>& tab, co
   }
   __syncthreads();
   // ---- z-lines: gradient along z, quadrature-point operation, transposed z pass ----
-  // cells without per-point geometry are axis-aligned boxes: diagonal metric
-  ff g00, g01, g02, g11, g12, g22;
-  if (!GEN) {
-    g00 = geo.cellG[e * 6 + 0]; g11 = geo.cellG[e * 6 + 3]; g22 = geo.cellG[e * 6 + 5];
-  }
   const ff* ptC = geo.ptC + (size_t)e * NQ3;
   for (int l = ty; l < NQ * NQ; l += nty) {
     ff t[NQ], h2[NQ], o[NQ];
@@ -146,21 +133,15 @@ __device__ __forceinline__ void cell_body_ff(const EOTables<ff, NP, NQ>& tab, co
       const ff d2 = h2[q];
       const int Q = q * NQ * NQ + l;
       const ff d0 = S0[Q * B + v], d1 = S1[Q * B + v];
-      if (GEN) {
-        const ff* pg = geo.ptG + (size_t)e * 6 * NQ3 + Q;
-        g00 = pg[0]; g01 = pg[NQ3]; g02 = pg[2 * NQ3]; g11 = pg[3 * NQ3]; g12 = pg[4 * NQ3]; g22 = pg[5 * NQ3];
-        ffacc r0 = acc_first(g00, d0), r1 = acc_first(g01, d0), r2 = acc_first(g02, d0);
-        acc_fma(r0, g01, d1); acc_fma(r0, g02, d2);
-        acc_fma(r1, g11, d1); acc_fma(r1, g12, d2);
-        acc_fma(r2, g12, d1); acc_fma(r2, g22, d2);
-        S0[Q * B + v] = acc_value(r0);
-        S1[Q * B + v] = acc_value(r1);
-        h2[q] = acc_value(r2);
-      } else {
-        S0[Q * B + v] = ff_mul(g00, d0);
-        S1[Q * B + v] = ff_mul(g11, d1);
-        h2[q] = ff_mul(g22, d2);
-      }
+      const ff* pg = geo.ptG + (size_t)e * 6 * NQ3 + Q;
+      const ff g00 = pg[0], g01 = pg[NQ3], g02 = pg[2 * NQ3], g11 = pg[3 * NQ3], g12 = pg[4 * NQ3], g22 = pg[5 * NQ3];
+      ffacc r0 = acc_first(g00, d0), r1 = acc_first(g01, d0), r2 = acc_first(g02, d0);
+      acc_fma(r0, g01, d1); acc_fma(r0, g02, d2);
+      acc_fma(r1, g11, d1); acc_fma(r1, g12, d2);
+      acc_fma(r2, g12, d1); acc_fma(r2, g22, d2);
+      S0[Q * B + v] = acc_value(r0);
+      S1[Q * B + v] = acc_value(r1);
+      h2[q] = acc_value(r2);
       t[q] = ff_mul(ptC[Q], t[q]);
     }
     eo_apply_ff<NQ, NQ, -1>(tab.Dt, h2, o);
@@ -226,19 +207,10 @@ __device__ __forceinline__ void cell_body_ff(const EOTables<ff, NP, NQ>& tab, co
     const size_t row = (size_t)(gy + (size_t)m.Ny * gz) * m.Nx;
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
-      size_t node;
-      bool con, first;
-      if constexpr (MAP) {
-        const int code = __ldg(map + (size_t)e * NP * NP * NP + l * NP + i);
-        node = (size_t)(code & kMapIndex);
-        con = (code & kMapConstrained) != 0;
-        first = (code & kMapFirst) != 0;
-      } else {
-        const int gx = node_coord(cx, i, P, m.Nx, m.periodic);
-        node = row + gx;
-        con = con_yz || on_boundary(gx, m.Nx, m.periodic);
-        first = first_yz && first_along(cx, m.nx, i, P, m.periodic, m.last_odd_x);
-      }
+      const int gx = node_coord(cx, i, P, m.Nx, m.periodic);
+      const size_t node = row + gx;
+      const bool con = con_yz || on_boundary(gx, m.Nx, m.periodic);
+      const bool first = first_yz && first_along(cx, m.nx, i, P, m.periodic, m.last_odd_x);
       double* dst = Y + node * n_vec + vg;
       if constexpr (SC) {
         scaled_store(dst, X + node * n_vec + vg, sc.a * __ldg(sc.msq + node) * ff_to_double(o[i]), first, con, sc);
@@ -250,22 +222,21 @@ __device__ __forceinline__ void cell_body_ff(const EOTables<ff, NP, NQ>& tab, co
   }
 }
 
-template <int NP, int NQ, bool GEN, bool SC, bool MAP>
+template <int NP, int NQ, bool SC>
 __global__ void __launch_bounds__(256) cell_apply_df64_kernel(const EOTables<ff, NP, NQ> tab, const MeshDev m,
                                                               const Geom<ff> geo, const int* __restrict__ cells,
                                                               int n_vec, int n_vb, const double* __restrict__ X,
-                                                              double* __restrict__ Y, const Scale<double> sc,
-                                                              const int* __restrict__ map) {
+                                                              double* __restrict__ Y, const Scale<double> sc) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cell_body_ff<NP, NQ, GEN, SC, MAP>(tab, m, geo, cells[blockIdx.x / n_vb], blockIdx.x % n_vb, blockDim.x,
+  cell_body_ff<NP, NQ, SC>(tab, m, geo, cells[blockIdx.x / n_vb], blockIdx.x % n_vb, blockDim.x,
                                      threadIdx.x, threadIdx.y, blockDim.y, n_vec, X, Y,
-                                     reinterpret_cast<ff*>(smem_raw), sc, map);
+                                     reinterpret_cast<ff*>(smem_raw), sc);
 }
 
-template <int NP, int NQ, bool GEN, bool SC, bool MAP = false>
+template <int NP, int NQ, bool SC>
 cudaError_t launch_df64(const fe_ctx* c, const double* X, double* Y, int n_vec, cudaStream_t s,
                         const Scale<double>& sc) {
-  auto kern = cell_apply_df64_kernel<NP, NQ, GEN, SC, MAP>;
+  auto kern = cell_apply_df64_kernel<NP, NQ, SC>;
   const int vb = pick_vb<double, NQ>(c->vbdf, n_vec);   // ff tiles take the bytes of FP64 tiles
   int nty = c->ntydf;
   if (vb * nty > 256) nty = 256 / vb;
@@ -284,7 +255,7 @@ cudaError_t launch_df64(const fe_ctx* c, const double* X, double* Y, int n_vec, 
     const long long blocks = (long long)n * n_vb;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     kern<<<(unsigned)blocks, dim3(vb, nty), smem, s>>>(tab, c->mdev, geo, c->d_cells + c->colors.offset[k], n_vec,
-                                                       n_vb, X, Y, sc, c->d_map);
+                                                       n_vb, X, Y, sc);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }

@@ -104,7 +104,11 @@ extern "C" fe_status fe_setup_refined(const fe_refined_desc* md, int p, const fe
   const int np = c->np, nq = c->nq, NP3 = np * np * np;
   const double* g = c->gll.data();
   double H[3];
-  for (int d = 0; d < 3; ++d) H[d] = (md->hi[d] - md->lo[d]) / n[d];
+  for (int d = 0; d < 3; ++d) {
+    H[d] = (md->hi[d] - md->lo[d]) / n[d];
+    c->box_lo[d] = md->lo[d];
+    c->box_h[d] = H[d];   // coarse cells; fine cells have the same aspect
+  }
   auto refined = [&](int cx, int cy, int cz) {
     return cx >= md->refine_lo[0] && cx < md->refine_hi[0] && cy >= md->refine_lo[1] && cy < md->refine_hi[1] &&
            cz >= md->refine_lo[2] && cz < md->refine_hi[2];
