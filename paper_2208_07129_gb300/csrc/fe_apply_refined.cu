@@ -57,14 +57,14 @@ cudaError_t cells_refined(const fe_ctx* c, const void* X, void* Y, int n_vec, cu
 #define FE_CASE(P, NQ)                                                                                       \
   if (c->p == P && c->nq == NQ) {                                                                            \
     if (c->mode == FE_FP32)                                                                                  \
-      return launch_box<float, P + 1, NQ, false, true>(c, static_cast<const float*>(X), static_cast<float*>(Y), \
-                                                       n_vec, s, c->vb32, c->nty32, make_geom<float>(c));    \
+      return launch_box<F2, P + 1, NQ, false, true>(c, static_cast<const float*>(X), static_cast<float*>(Y), \
+                                                       n_vec, s, c->tile32(), make_geom<float>(c));            \
     const double* X64 = static_cast<const double*>(X);                                                       \
     double* Y64 = static_cast<double*>(Y);                                                                   \
     return c->mode == FE_FP64                                                                                \
-               ? launch_box<double, P + 1, NQ, false, true>(c, X64, Y64, n_vec, s, c->vb64, c->nty64,        \
+               ? launch_box<double, P + 1, NQ, false, true>(c, X64, Y64, n_vec, s, c->tile64(),               \
                                                             make_geom<double>(c))                            \
-               : launch_box<ff, P + 1, NQ, false, true>(c, X64, Y64, n_vec, s, c->vbdf, c->ntydf, make_geom<ff>(c)); \
+               : launch_box<ff, P + 1, NQ, false, true>(c, X64, Y64, n_vec, s, c->tiledf(), make_geom<ff>(c)); \
   }
   FE_FOR_EACH_P_NQ(FE_CASE)
 #undef FE_CASE

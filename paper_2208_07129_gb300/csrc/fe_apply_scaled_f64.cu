@@ -10,7 +10,7 @@ cudaError_t apply_scaled_f64(const fe_ctx* c, const double* X, double* Y, int n_
 #define FE_CASE(P, NQ)                                                                                        \
   if (c->p == P && c->nq == NQ)                                                                         \
     return c->general ? launch_apply_eo<double, P + 1, NQ, true>(c, X, Y, n_vec, s, c->vb64, c->nty64, sc)  \
-                      : launch_box<double, P + 1, NQ, true>(c, X, Y, n_vec, s, c->vb64, c->nty64, make_geom<double>(c), sc);
+                      : launch_box<double, P + 1, NQ, true>(c, X, Y, n_vec, s, c->tile64(), make_geom<double>(c), sc);
   FE_FOR_EACH_P_NQ(FE_CASE)
 #undef FE_CASE
   return cudaErrorInvalidValue;

@@ -38,10 +38,10 @@ constexpr int kTabImage = 256;   // elements of a BoxTables<T, NP, NQ> image (24
 template <typename T>
 struct BatchProblemDev {
   MeshDev m;
-  Geom<T> geo;
-  int n_vec, vb, nty, kind, n_vb;
+  Geom<typename Arith<T>::G> geo;
+  int n_vec, vb, nty, kind, n_vb;                      // vb: vectors per item
   const int* cells;                                    // colour-sorted cell ids
-  T tab[kTabImage];                                    // BoxTables<T, NP, NQ> image
+  typename Arith<T>::C tab[kTabImage];                                    // BoxTables<T, NP, NQ> image
 };
 
 struct WorkItem {
@@ -54,12 +54,13 @@ constexpr int kind_of(int p) { return p - 3; }
 template <typename T, int NP, int NQ>
 __device__ __forceinline__ void run_item(const BatchProblemDev<T>& P, const WorkItem& w,
                                          const typename Arith<T>::D* X, typename Arith<T>::D* Y, T* smem,
-                                         const BoxTables<T, NP, NQ>& tab) {
-  const int tid = threadIdx.x, vb = P.vb;
-  const int v = tid % vb, ty = tid / vb, nty = kBatchThreads / vb;
+                                         const BoxTables<typename Arith<T>::C, NP, NQ>& tab) {
+  const int tid = threadIdx.x, lanes = P.vb / Arith<T>::W;
+  const int v = tid % lanes, ty = tid / lanes, nty = kBatchThreads / lanes;
+  const bool vec = vec_ok<T>(X, Y, P.n_vec);
   for (int c = 0; c < w.cell_count; ++c) {
     const int e = P.cells[w.cell_begin + c];
-    cell_body_box<T, NP, NQ>(tab, P.m, P.geo, e, w.vb, vb, v, ty, nty, P.n_vec, X, Y, smem,
+    cell_body_box<T, NP, NQ>(tab, P.m, P.geo, e, w.vb, lanes, v, ty, nty, P.n_vec, vec, X, Y, smem,
                              Scale<typename Arith<T>::D>{});
     __syncthreads();
   }
@@ -78,7 +79,7 @@ __device__ __forceinline__ unsigned long long batch_clock_ns() {
 // contractions read their coefficients from the constant bank as in the
 // per-colour kernels.
 template <typename T, int NP, int NQ>
-__global__ void __launch_bounds__(kBatchThreads) batch_kernel(const BoxTables<T, NP, NQ> tab,
+__global__ void __launch_bounds__(kBatchThreads) batch_kernel(const BoxTables<typename Arith<T>::C, NP, NQ> tab,
                                                              const BatchProblemDev<T>* __restrict__ probs,
                                                              const void* const* __restrict__ ptrs,
                                                              const WorkItem* __restrict__ items, int n_items,
@@ -134,7 +135,7 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel_all(const BatchPro
                                                                  int* next, int* done, const int* __restrict__ need,
                                                                  int* status, const long long* __restrict__ wait_ns) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ __align__(16) T stab[kTabImage];
+  __shared__ __align__(16) typename Arith<T>::C stab[kTabImage];
   __shared__ int s_item;
   T* smem = reinterpret_cast<T*>(smem_raw);
   for (;;) {
@@ -163,7 +164,7 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel_all(const BatchPro
     const D* X = static_cast<const D*>(ptrs[2 * w.problem]);
     D* Y = static_cast<D*>(const_cast<void*>(ptrs[2 * w.problem + 1]));
 #define FE_ITEM(K, NP, NQ) \
-  case K: run_item<T, NP, NQ>(P, w, X, Y, smem, *reinterpret_cast<const BoxTables<T, NP, NQ>*>(stab)); break;
+  case K: run_item<T, NP, NQ>(P, w, X, Y, smem, *reinterpret_cast<const BoxTables<typename Arith<T>::C, NP, NQ>*>(stab)); break;
     switch (P.kind) {
       FE_ITEM(0, 4, 5) FE_ITEM(1, 5, 6) FE_ITEM(2, 6, 7) FE_ITEM(3, 7, 8) FE_ITEM(4, 8, 9) FE_ITEM(5, 9, 10)
       default: break;
@@ -219,17 +220,19 @@ fe_status from_cuda(cudaError_t e) {
 
 template <typename T>
 size_t tile_smem(int nq, int vb) {
-  const int pitch[] = {0, 0, BoxTile<2>::pitch(vb), BoxTile<3>::pitch(vb), BoxTile<4>::pitch(vb), BoxTile<5>::pitch(vb),
-                       BoxTile<6>::pitch(vb), BoxTile<7>::pitch(vb), BoxTile<8>::pitch(vb), BoxTile<9>::pitch(vb),
-                       BoxTile<10>::pitch(vb)};
-  return (size_t)2 * vb * pitch[nq] * sizeof(T);
+  const int B = vb / Arith<T>::W, U = (int)sizeof(T);
+  const int pitch[] = {0, 0, BoxTile<2>::pitch(B, U), BoxTile<3>::pitch(B, U), BoxTile<4>::pitch(B, U),
+                       BoxTile<5>::pitch(B, U), BoxTile<6>::pitch(B, U), BoxTile<7>::pitch(B, U),
+                       BoxTile<8>::pitch(B, U), BoxTile<9>::pitch(B, U), BoxTile<10>::pitch(B, U)};
+  return (size_t)2 * B * pitch[nq] * sizeof(T);
 }
 
 // The tables of one problem, copied into its table image.
 template <typename T, int NP, int NQ>
-void box_image(const fe_ctx* c, T* img) {
-  static_assert(sizeof(BoxTables<T, NP, NQ>) <= kTabImage * sizeof(T), "table image too small");
-  const BoxTables<T, NP, NQ> t = make_boxtables<T, NP, NQ>(c);
+void box_image(const fe_ctx* c, typename Arith<T>::C* img) {
+  using C = typename Arith<T>::C;
+  static_assert(sizeof(BoxTables<C, NP, NQ>) <= kTabImage * sizeof(C), "table image too small");
+  const BoxTables<C, NP, NQ> t = make_boxtables<C, NP, NQ>(c);
   std::memcpy(img, &t, sizeof(t));
 }
 
@@ -275,7 +278,7 @@ int autotune(const fe_ctx* c, int n_vec_full, fe_mode mode, float* spent_ms) {
     cudaEventCreate(&b);
     float best_ms = 1e30f;
     for (int vb : cand) {
-      fe_set_tile(px, mode, vb, kBatchThreads / vb, mode == FE_FP32 ? 3 : 0);   // the box-cell kernel
+      fe_set_tile(px, mode, vb, kBatchThreads / (vb / Arith<T>::W), mode == FE_FP32 ? 3 : 0);   // the box-cell kernel
       fe_apply(px, X, Y, n_vec, nullptr);
       cudaEventRecord(a);
       for (int r = 0; r < 3; ++r) fe_apply(px, X, Y, n_vec, nullptr);
@@ -316,7 +319,8 @@ cudaError_t prepare_group(fe_batch* b, int g, int n_g, size_t smem) {
 template <typename T, int NP, int NQ>
 cudaError_t launch_group(fe_batch* b, int g, int n_g, size_t smem) {
   auto kern = batch_kernel<T, NP, NQ>;
-  const BoxTables<T, NP, NQ> tab = make_boxtables<T, NP, NQ>(b->ctxs[b->group_first[g]]);
+  using C = typename Arith<T>::C;
+  const BoxTables<C, NP, NQ> tab = make_boxtables<C, NP, NQ>(b->ctxs[b->group_first[g]]);
   kern<<<b->group_grid[g], kBatchThreads, smem, b->side[g]>>>(
       tab, static_cast<const BatchProblemDev<T>*>(b->d_probs), const_cast<const void* const*>(b->d_ptrs),
       b->d_items + b->item_begin[g], n_g, b->d_next + g, b->d_done, b->d_need, b->d_status, b->d_wait_ns);
@@ -358,9 +362,7 @@ fe_status build_batch(fe_batch* b, int autotune_on) {
     fe_ctx* c = b->ctxs[i];
     BatchProblemDev<T>& P = hp[i];
     P.m = c->mdev;
-    if constexpr (std::is_same<T, ff>::value) P.geo = Geom<ff>{c->d_cellGff, c->d_ptGff, c->d_ptCff};
-    else if (b->mode == FE_FP64) P.geo = Geom<T>{(const T*)c->d_cellG64, (const T*)c->d_ptG64, (const T*)c->d_ptC64};
-    else P.geo = Geom<T>{(const T*)c->d_cellG32, (const T*)c->d_ptG32, (const T*)c->d_ptC32};
+    P.geo = make_geom<typename Arith<T>::G>(c);
     P.n_vec = b->n_vec[i];
     P.kind = kind_of(c->p);
     P.cells = c->d_cells;
@@ -545,7 +547,7 @@ extern "C" fe_status fe_batch_create(fe_ctx* const* ctxs, int n, const int* n_ve
   b->cells_per_item.assign(n, 1);
   fe_status st = mode == FE_FP64 ? build_batch<double>(b, autotune_on)
                  : mode == FE_DF64 ? build_batch<ff>(b, autotune_on)
-                                   : build_batch<float>(b, autotune_on);
+                                   : build_batch<F2>(b, autotune_on);
   if (st != FE_OK) {
     fe_batch_destroy(b);
     return st;

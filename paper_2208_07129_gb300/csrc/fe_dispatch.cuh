@@ -8,6 +8,33 @@
 
 namespace fe {
 
+// The colour launches of one product overlap: a launch made with `overlap` may
+// start as soon as every CTA of the one before it has started (programmatic
+// dependent launch), and its CTAs gather and contract their cells while the
+// earlier colour finishes.  They touch Y only after wait_for_earlier_launch(),
+// which returns once the earlier launch has completed (and with it, since
+// each launch waits in the same way, all before it).  A product's first
+// launch is an ordinary one.
+__device__ __forceinline__ void let_next_launch_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_earlier_launch() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... P, typename... Args>
+cudaError_t launch_kernel(void (*kern)(P...), size_t blocks, dim3 threads, size_t smem, cudaStream_t s, bool overlap,
+                          Args... args) {
+  if (blocks > 0x7fffffffull) return cudaErrorInvalidConfiguration;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = threads;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 template <typename T, int NP, int NQ>
 Tables<T, NP, NQ> make_tables(const fe_ctx* c) {
   Tables<T, NP, NQ> t;

@@ -205,6 +205,7 @@ __device__ __forceinline__ void cell_body_eo(const EOTables<T, NP, NQ>& tab, con
   }
   __syncthreads();
   // ---- transposed x pass of N fused with assembly ----
+  if constexpr (!LOCAL) wait_for_earlier_launch();
   for (int l = ty; l < NP * NP; l += nty) {
     const int i2 = l % NP, i3 = l / NP;
     T t[NQ], o[NP];
@@ -246,6 +247,7 @@ __global__ void __launch_bounds__(256) cell_apply_eo_kernel(const EOTables<T, NP
                                                             int n_vec, int n_vb, const T* __restrict__ X,
                                                             T* __restrict__ Y) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  let_next_launch_start();
   cell_body_eo<T, NP, NQ>(tab, m, geo, cells[blockIdx.x / n_vb], blockIdx.x % n_vb, blockDim.x, threadIdx.x,
                                threadIdx.y, blockDim.y, n_vec, X, Y, reinterpret_cast<T*>(smem_raw));
 }
@@ -257,6 +259,7 @@ __global__ void __launch_bounds__(256) cell_apply_eo_scaled_kernel(const EOTable
                                                                    int n_vec, int n_vb, const T* __restrict__ X,
                                                                    T* __restrict__ Y, const Scale<T> sc) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  let_next_launch_start();
   cell_body_eo<T, NP, NQ, true>(tab, m, geo, cells[blockIdx.x / n_vb], blockIdx.x % n_vb, blockDim.x,
                                      threadIdx.x, threadIdx.y, blockDim.y, n_vec, X, Y,
                                      reinterpret_cast<T*>(smem_raw), sc);
@@ -268,6 +271,7 @@ __global__ void __launch_bounds__(256) cell_apply_eo_local_kernel(const EOTables
                                                                   const Geom<T> geo, int n_vec, int n_vb,
                                                                   const T* __restrict__ X, T* __restrict__ W) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  let_next_launch_start();
   cell_body_eo<T, NP, NQ, false, true>(tab, m, geo, blockIdx.x / n_vb, blockIdx.x % n_vb, blockDim.x,
                                                    threadIdx.x, threadIdx.y, blockDim.y, n_vec, X, W,
                                                    reinterpret_cast<T*>(smem_raw));
@@ -305,6 +309,7 @@ __global__ void assemble_local_kernel(const MeshDev m, const T* __restrict__ W, 
                                       int n_vec) {
   constexpr int P = NP - 1, NP3 = NP * NP * NP;
   const size_t total = n_dofs * n_vec;
+  wait_for_earlier_launch();
   for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
        idx += (size_t)gridDim.x * blockDim.x) {
     const size_t dof = idx / n_vec;
@@ -389,28 +394,29 @@ cudaError_t launch_apply_eo(const fe_ctx* c, const T* X, T* Y, int n_vec, cudaSt
       cudaError_t e = ensure_dyn_smem(reinterpret_cast<const void*>(lk), lsm);
       if (e != cudaSuccess) return e;
       T* W = static_cast<T*>(c->d_small);
-      lk<<<(unsigned)(c->n_cells * (size_t)n_vec), dim3(1, lines), lsm, s>>>(tab, c->mdev, geo, n_vec, n_vec, X, W);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      e = launch_kernel(lk, c->n_cells * (size_t)n_vec, dim3(1, lines), lsm, s, false, tab, c->mdev, geo, n_vec, n_vec, X,
+                        W);
+      if (e != cudaSuccess) return e;
       const size_t tot = c->n_dofs * (size_t)n_vec;
-      assemble_local_kernel<T, NP><<<(unsigned)std::min<size_t>((tot + 255) / 256, 152 * 8), 256, 0, s>>>(
-          c->mdev, W, Y, c->n_dofs, n_vec);
-      return cudaGetLastError();
+      return launch_kernel(assemble_local_kernel<T, NP>, std::min<size_t>((tot + 255) / 256, 152 * 8), dim3(256), 0, s,
+                           true, c->mdev, W, Y, c->n_dofs, n_vec);
     }
   }
   const int n_vb = (n_vec + vb - 1) / vb;
+  bool overlap = false;
   for (int k = 0; k < c->colors.n_colors; ++k) {
     const int n = c->colors.offset[k + 1] - c->colors.offset[k];
     if (n == 0) continue;
-    const long long blocks = (long long)n * n_vb;
-    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    const int* cells = c->d_cells + c->colors.offset[k];
+    cudaError_t e;
     if constexpr (SC)
-      cell_apply_eo_scaled_kernel<T, NP, NQ><<<(unsigned)blocks, dim3(vb, nty), smem, s>>>(
-          tab, c->mdev, geo, c->d_cells + c->colors.offset[k], n_vec, n_vb, X, Y, sc);
+      e = launch_kernel(cell_apply_eo_scaled_kernel<T, NP, NQ>, (size_t)n * n_vb, dim3(vb, nty), smem, s, overlap, tab,
+                        c->mdev, geo, cells, n_vec, n_vb, X, Y, sc);
     else
-      cell_apply_eo_kernel<T, NP, NQ><<<(unsigned)blocks, dim3(vb, nty), smem, s>>>(
-          tab, c->mdev, geo, c->d_cells + c->colors.offset[k], n_vec, n_vb, X, Y);
-    cudaError_t e = cudaGetLastError();
+      e = launch_kernel(cell_apply_eo_kernel<T, NP, NQ>, (size_t)n * n_vb, dim3(vb, nty), smem, s, overlap, tab, c->mdev,
+                        geo, cells, n_vec, n_vb, X, Y);
     if (e != cudaSuccess) return e;
+    overlap = true;
   }
   return cudaSuccess;
 }

@@ -193,6 +193,7 @@ __device__ __forceinline__ void cell_body_ff(const EOTables<ff, NP, NQ>& tab, co
   }
   __syncthreads();
   // ---- transposed x pass of N fused with assembly (FP64) ----
+  wait_for_earlier_launch();
   for (int l = ty; l < NP * NP; l += nty) {
     const int i2 = l % NP, i3 = l / NP;
     ff t[NQ], o[NP];
@@ -228,6 +229,7 @@ __global__ void __launch_bounds__(256) cell_apply_df64_kernel(const EOTables<ff,
                                                               int n_vec, int n_vb, const double* __restrict__ X,
                                                               double* __restrict__ Y, const Scale<double> sc) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  let_next_launch_start();
   cell_body_ff<NP, NQ, SC>(tab, m, geo, cells[blockIdx.x / n_vb], blockIdx.x % n_vb, blockDim.x,
                                      threadIdx.x, threadIdx.y, blockDim.y, n_vec, X, Y,
                                      reinterpret_cast<ff*>(smem_raw), sc);
@@ -249,15 +251,14 @@ cudaError_t launch_df64(const fe_ctx* c, const double* X, double* Y, int n_vec, 
   const EOTables<ff, NP, NQ> tab = make_eotables<ff, NP, NQ>(c);
   const Geom<ff> geo{c->d_cellGff, c->d_ptGff, c->d_ptCff};
   const int n_vb = (n_vec + vb - 1) / vb;
+  bool overlap = false;
   for (int k = 0; k < c->colors.n_colors; ++k) {
     const int n = c->colors.offset[k + 1] - c->colors.offset[k];
     if (n == 0) continue;
-    const long long blocks = (long long)n * n_vb;
-    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    kern<<<(unsigned)blocks, dim3(vb, nty), smem, s>>>(tab, c->mdev, geo, c->d_cells + c->colors.offset[k], n_vec,
-                                                       n_vb, X, Y, sc);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_kernel(kern, (size_t)n * n_vb, dim3(vb, nty), smem, s, overlap, tab, c->mdev, geo,
+                                        c->d_cells + c->colors.offset[k], n_vec, n_vb, X, Y, sc);
     if (e != cudaSuccess) return e;
+    overlap = true;
   }
   return cudaSuccess;
 }

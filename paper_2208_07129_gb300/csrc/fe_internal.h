@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "../../include/fe.h"
+#include "fe_arith.cuh"
 #include "fe_ff.cuh"
 
 namespace fe {
@@ -110,6 +111,9 @@ struct fe_ctx {
   // host FP64 data
   std::vector<double> gll, wgll, qx, qw, N1, D1;   // N1[q*np+i], D1[q*nq+k] (unfolded)
   std::vector<double> Nf, Df;                // folded
+  // stiffness at the points, K = Df^T Df: K[i][j] + K[i][nq-1-j] and the
+  // difference, i < (nq+1)/2, j < nq/2, then the middle column (box kernel)
+  std::vector<double> Ks, Kd;
   std::vector<double> vertices;              // copy of the vertex array (general)
   double box_lo[3] = {0, 0, 0}, box_h[3] = {1, 1, 1};  // uniform box: corner and cell size
   std::vector<double> detJ;                  // per point (E*nq3)
@@ -164,6 +168,11 @@ struct fe_ctx {
   void* solver = nullptr;
   // launch shape per mode (vectors per CTA, lines per CTA)
   int vb64 = 8, nty64 = 16, vb32 = 8, nty32 = 32, vbdf = 8, ntydf = 32;
+  // the box kernel has its own defaults (Arith::box_tile) until fe_set_tile sets a tile
+  bool set64 = false, set32 = false, setdf = false;
+  fe::LineTile tile64() const { return set64 ? fe::LineTile{vb64, nty64} : fe::LineTile{0, 0}; }
+  fe::LineTile tile32() const { return set32 ? fe::LineTile{vb32, nty32} : fe::LineTile{0, 0}; }
+  fe::LineTile tiledf() const { return setdf ? fe::LineTile{vbdf, ntydf} : fe::LineTile{0, 0}; }
   int fp32_variant = 0;   // 0 / 1: line kernel, 2: register-plane kernel, 3: even-odd line kernel
   int fp64_variant = 0;   // 0: even-odd line kernel, 1: plain line kernel
   int tc_variant = 0;     // FE_TF32 / FE_BF16 / FE_BF16S: 0 tcgen05 kernel (where built) with TMA boxes where

@@ -167,6 +167,8 @@ cudaError_t upload_as_ff(ff** dst, const std::vector<double>& src) {
 
 }  // namespace
 
+static void build_stiffness(fe_ctx* c);
+
 // GLL nodes and weights (n_p points), the quadrature rule, and the 1D
 // tables: N (values at the points) and D~ (collocation derivative), plain
 // and with sqrt(w) folded in (Sec. 3.2.4).  Needs c->np, c->nq, c->quad_kind.
@@ -186,6 +188,27 @@ void build_tables(fe_ctx* c) {
       c->D1[q * nq + k] = lagrange_deriv(c->qx.data(), nq, k, c->qx[q]);
       c->Df[q * nq + k] = c->D1[q * nq + k] * std::sqrt(c->qw[q] / c->qw[k]);
     }
+  }
+  build_stiffness(c);
+}
+
+// Ks, Kd: extended precision, so that forming the matrix adds one rounding to
+// those of the folded table.
+static void build_stiffness(fe_ctx* c) {
+  const int nq = c->nq, HE = (nq + 1) / 2, H = nq / 2;
+  auto k = [&](int a, int b) {
+    long double s = 0.0L;
+    for (int q = 0; q < nq; ++q) s += (long double)c->Df[q * nq + a] * c->Df[q * nq + b];
+    return s;
+  };
+  c->Ks.assign((size_t)HE * HE, 0.0);
+  c->Kd.assign((size_t)HE * HE, 0.0);
+  for (int o = 0; o < HE; ++o) {
+    for (int i = 0; i < H; ++i) {
+      c->Ks[o * HE + i] = (double)(k(o, i) + k(o, nq - 1 - i));
+      c->Kd[o * HE + i] = (double)(k(o, i) - k(o, nq - 1 - i));
+    }
+    if (HE > H) c->Ks[o * HE + H] = (double)k(o, H);
   }
 }
 
@@ -503,15 +526,18 @@ extern "C" fe_status fe_set_tile(fe_ctx* c, fe_mode mode, int vectors_per_cta, i
     if (variant >= 2) return FE_EINVAL;
     c->vb64 = vectors_per_cta;
     c->nty64 = lines;
+    c->set64 = true;
     c->fp64_variant = variant;
   } else if (mode == FE_DF64) {
     if (variant != 0) return FE_EINVAL;
     c->vbdf = vectors_per_cta;
     c->ntydf = lines;
+    c->setdf = true;
   } else if (mode == FE_FP32) {
     if (variant == 2 && c->nq > 8) return FE_EUNSUPPORTED;
     c->vb32 = vectors_per_cta;
     c->nty32 = lines;
+    c->set32 = true;
     c->fp32_variant = variant;
   } else if (mode == FE_TF32 || mode == FE_BF16) {
     if (variant > 2) return FE_EINVAL;   // tensor-core tiles are fixed: only the kernel is chosen
