@@ -3,6 +3,7 @@
 // selected with fe_set_tile.
 #include "fe_dispatch.cuh"
 #include "fe_box.cuh"
+#include "fe_general.cuh"
 #include "fe_plane_kernel.cuh"
 
 namespace fe {
@@ -14,7 +15,7 @@ cudaError_t pick(const fe_ctx* c, const float* X, float* Y, int n_vec, cudaStrea
     if (c->fp32_variant == 2) return launch_plane<NP, NQ, GEN>(c, X, Y, n_vec, s);
   }
   if (c->fp32_variant == 3) {
-    if constexpr (GEN) return launch_apply_eo<float, NP, NQ>(c, X, Y, n_vec, s, c->vb32, c->nty32);
+    if constexpr (GEN) return launch_general<F2, NP, NQ>(c, X, Y, n_vec, s, c->tile32(), make_geom<float>(c));
     else return launch_box<F2, NP, NQ>(c, X, Y, n_vec, s, c->tile32(), make_geom<float>(c));
   }
   return launch_apply<float, NP, NQ, GEN>(c, X, Y, n_vec, s, c->vb32, c->nty32);

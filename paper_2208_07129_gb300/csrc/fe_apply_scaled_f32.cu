@@ -2,6 +2,7 @@
 // Y = a M^-1/2 A M^-1/2 X + b X + c Y (even-odd line kernel).
 #include "fe_dispatch.cuh"
 #include "fe_box.cuh"
+#include "fe_general.cuh"
 
 namespace fe {
 
@@ -9,7 +10,7 @@ cudaError_t apply_scaled_f32(const fe_ctx* c, const float* X, float* Y, int n_ve
                              cudaStream_t s) {
 #define FE_CASE(P, NQ)                                                                                       \
   if (c->p == P && c->nq == NQ)                                                                         \
-    return c->general ? launch_apply_eo<float, P + 1, NQ, true>(c, X, Y, n_vec, s, c->vb32, c->nty32, sc)  \
+    return c->general ? launch_general<F2, P + 1, NQ, true>(c, X, Y, n_vec, s, c->tile32(), make_geom<float>(c), sc) \
                       : launch_box<F2, P + 1, NQ, true>(c, X, Y, n_vec, s, c->tile32(), make_geom<float>(c), sc);
   FE_FOR_EACH_P_NQ(FE_CASE)
 #undef FE_CASE

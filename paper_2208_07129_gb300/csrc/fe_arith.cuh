@@ -68,6 +68,10 @@ struct Arith<double> {
   static constexpr LineTile box_tile(int nq) {
     return nq <= 5 ? LineTile{32, 8} : nq <= 7 ? LineTile{16, 8} : nq == 8 ? LineTile{8, 16} : nq == 9 ? LineTile{8, 24} : LineTile{4, 32};
   }
+  // Default tile of the trilinear kernel (three tiles of shared memory), swept the same way.
+  static constexpr LineTile general_tile(int nq) {
+    return nq <= 5 ? LineTile{32, 8} : nq == 6 ? LineTile{16, 16} : nq <= 8 ? LineTile{8, 16} : LineTile{4, 32};
+  }
   static __device__ __forceinline__ V zero() { return 0.0; }
   static __device__ __forceinline__ V add(V a, V b) { return __dadd_rn(a, b); }
   static __device__ __forceinline__ V sub(V a, V b) { return __dsub_rn(a, b); }
@@ -75,6 +79,7 @@ struct Arith<double> {
   static __device__ __forceinline__ Acc init(V v) { return v; }
   static __device__ __forceinline__ void fma(Acc& a, C c, V v) { a = __fma_rn(c, v, a); }
   static __device__ __forceinline__ V value(Acc a) { return a; }
+  static __device__ __forceinline__ V muladd(G c, V v, V a) { return __fma_rn(c, v, a); }
   // c v + g s: the middle point of an odd rule
   static __device__ __forceinline__ V point(G c, V v, G g, V s) { return __fma_rn(g, s, __dmul_rn(c, v)); }
   // e = c1 v1 + c2 v2 + g se,  o = c1 v1 - c2 v2 + g so
@@ -144,6 +149,9 @@ struct Arith<F2> {
   static constexpr LineTile box_tile(int nq) {
     return nq <= 4 ? LineTile{32, 8} : nq <= 6 ? LineTile{16, 16} : nq <= 8 ? LineTile{16, 32} : LineTile{8, 32};
   }
+  static constexpr LineTile general_tile(int nq) {
+    return nq <= 4 ? LineTile{32, 8} : nq == 5 ? LineTile{16, 16} : nq <= 8 ? LineTile{8, 32} : LineTile{8, 40};
+  }
   static __device__ __forceinline__ V zero() { return V{0ull}; }
   static __device__ __forceinline__ V add(V a, V b) { return V{add2(a.v, b.v)}; }
   static __device__ __forceinline__ V sub(V a, V b) { return V{sub2(a.v, b.v)}; }
@@ -151,6 +159,7 @@ struct Arith<F2> {
   static __device__ __forceinline__ Acc init(V v) { return v.v; }
   static __device__ __forceinline__ void fma(Acc& a, C c, V v) { a = fma2(bc(c), v.v, a); }
   static __device__ __forceinline__ V value(Acc a) { return V{a}; }
+  static __device__ __forceinline__ V muladd(G c, V v, V a) { return V{fma2(bc(c), v.v, a.v)}; }
   static __device__ __forceinline__ V point(G c, V v, G g, V s) { return V{fma2(bc(g), s.v, mul2(bc(c), v.v))}; }
   static __device__ __forceinline__ void point_pair(G c1, V v1, G c2, V v2, G g, V se, V so, V& e, V& o) {
     const f32x2 gg = bc(g), p = mul2(bc(c1), v1.v);
@@ -181,6 +190,9 @@ struct Arith<ff> {
   static constexpr LineTile box_tile(int nq) {
     return nq <= 5 ? LineTile{16, 8} : nq <= 7 ? LineTile{16, 16} : nq <= 9 ? LineTile{8, 32} : LineTile{4, 64};
   }
+  static constexpr LineTile general_tile(int nq) {
+    return nq <= 4 ? LineTile{16, 8} : nq <= 6 ? LineTile{16, 16} : nq <= 8 ? LineTile{8, 32} : LineTile{4, 32};
+  }
   static __device__ __forceinline__ V zero() { return ff(0.f, 0.f); }
   static __device__ __forceinline__ V add(V a, V b) { return ff_add(a, b); }
   static __device__ __forceinline__ V sub(V a, V b) { return ff_sub(a, b); }
@@ -188,6 +200,7 @@ struct Arith<ff> {
   static __device__ __forceinline__ Acc init(V v) { return Acc{v.hi, v.lo}; }
   static __device__ __forceinline__ void fma(Acc& a, C c, V v) { acc_fma(a, c, v); }
   static __device__ __forceinline__ V value(const Acc& a) { return acc_value(a); }
+  static __device__ __forceinline__ V muladd(G c, V v, V a) { return ff_add(acc_value(acc_first(c, v)), a); }
   static __device__ __forceinline__ V point(G c, V v, G g, V s) {
     Acc a = acc_first(c, v);
     acc_fma(a, g, s);

@@ -6,14 +6,14 @@
 // points is separable,
 //   D~_x^T g00 D~_x + D~_y^T g11 D~_y + D~_z^T g22 D~_z,   and   D~^T D~ = K
 // is one symmetric n_q x n_q matrix: three 1D passes with K take the place of
-// the six passes with D~ and D~^T of trilinear cells (fe_evenodd.cuh), and
+// the six passes with D~ and D~^T of trilinear cells (fe_general.cuh), and
 // nothing but the values t = N u has to be kept besides their image s.  K is
 // formed in FP64 on the host; the cell's one factor g22 multiplies at the end
 // (g00 / g22 and g11 / g22 are the same for every cell of a mesh and are part
 // of the x and y tables).
 //
 // Each 1D matrix is (skew-)centrosymmetric, so it splits into an even and an
-// odd half (see fe_evenodd.cuh).  Here the halves stay apart between passes:
+// odd half (see fe_cells.cuh).  Here the halves stay apart between passes:
 // a direction's values are kept as (even, odd) parts from N's pass until the
 // pass that needs point values, so K works on them without sums before or
 // after.  For p = 6, n_q = 8 a cell and vector take 22.5 K operations against
@@ -29,16 +29,21 @@
 // The tiles hold one vector group after the other with constant strides, so
 // every access has an immediate offset; rows are padded to an odd length and
 // the distance of two groups is chosen so that no pass meets a bank conflict.
+//
+// What bounds it, and what it measured (32^3 periodic, p = 6, n_q = 8, 64
+// vectors; the D~ form before): FP64 148.0 -> 89.9 ms, the FP64 pipe (22.5 K
+// operations at 0.595 T/s are 79 ms); double-float 38.9 -> 20.9 ms, the issue
+// of FP32 instructions.  FP32, 24^3, 128 vectors: 6.92 -> 2.99 ms, shared
+// memory (7.5 K values per cell and vector, 1.2 ms) and the barriers between
+// the passes.
 #pragma once
 
-#include <algorithm>
-
-#include "fe_arith.cuh"
-#include "fe_evenodd.cuh"
+#include "fe_cells.cuh"
 
 namespace fe {
 
-// Tables of the box kernel for C coefficients.  N, Nt as in EOTables; K maps
+// Tables of the box kernel for C coefficients.  N: nodes to points, Nt its
+// transpose; K maps
 // (even, odd) parts to (even, odd) parts.
 template <typename C, int NP, int NQ>
 struct BoxTables {
@@ -47,116 +52,8 @@ struct BoxTables {
   EOTab<C, NQ, NQ> Kx, Ky, Kz;
 };
 
-// Sums and differences of mirrored values: in -> (even, odd).
-template <typename A, int N>
-__device__ __forceinline__ void eo_split(const typename A::V* in, typename A::V* e, typename A::V* o) {
-#pragma unroll
-  for (int i = 0; i < N / 2; ++i) {
-    e[i] = A::add(in[i], in[N - 1 - i]);
-    o[i] = A::sub(in[i], in[N - 1 - i]);
-  }
-  if constexpr (N & 1) e[N / 2] = in[N / 2];
-}
-
-// Values from their (even, odd) parts; part k is stored at index k of x
-// (even parts first), the values replace them.
-template <typename A, int N>
-__device__ __forceinline__ void eo_join(typename A::V* x) {
-  constexpr int H = N / 2, HE = (N + 1) / 2;
-  typename A::V t[N];
-#pragma unroll
-  for (int i = 0; i < H; ++i) {
-    t[i] = A::add(x[i], x[HE + i]);
-    t[N - 1 - i] = A::sub(x[i], x[HE + i]);
-  }
-  if constexpr (N & 1) t[H] = x[H];
-#pragma unroll
-  for (int i = 0; i < N; ++i) x[i] = t[i];
-}
-
-// out parts = tables times in parts (even parts first in out); with ADD the
-// products are added to what out holds.  Double-float and FP32 sum the products
-// first and add the sum: what out holds is larger than one direction's share,
-// and every term added to it would be rounded at its scale (the double-float
-// error of a p = 6 product is 1.2e-14 this way, 1.4e-14 the other).  FP64
-// starts its sum from it: one operation less on the pipe that bounds it.
-template <typename A, int NI, typename TC, typename TV>
-__device__ __forceinline__ typename A::V eo_dot(const TC* c, const TV* x) {
-  typename A::Acc a = A::first(c[0], x[0]);
-#pragma unroll
-  for (int i = 1; i < NI; ++i) A::fma(a, c[i], x[i]);
-  return A::value(a);
-}
-
-template <typename A, int NI, bool ADD, typename TC>
-__device__ __forceinline__ void eo_row(const TC* c, const typename A::V* x, typename A::V& out) {
-  if constexpr (!ADD) {
-    out = eo_dot<A, NI>(c, x);
-  } else if constexpr (A::kSumApart) {
-    out = A::add(out, eo_dot<A, NI>(c, x));
-  } else {
-    typename A::Acc a = A::init(out);
-#pragma unroll
-    for (int i = 0; i < NI; ++i) A::fma(a, c[i], x[i]);
-    out = A::value(a);
-  }
-}
-
-template <typename A, int NO, int NI, bool ADD = false>
-__device__ __forceinline__ void eo_parts(const EOTab<typename A::C, NO, NI>& t, const typename A::V* e,
-                                         const typename A::V* o, typename A::V* out) {
-  constexpr int HI = NI / 2, HE = (NI + 1) / 2, HO = (NO + 1) / 2;
-#pragma unroll
-  for (int k = 0; k < HO; ++k) eo_row<A, HE, ADD>(t.E[k], e, out[k]);
-#pragma unroll
-  for (int k = 0; k < NO / 2; ++k) {
-    if constexpr (HI > 0) eo_row<A, HI, ADD>(t.O[k], o, out[HO + k]);
-    else if (!ADD) out[HO + k] = A::zero();
-  }
-}
-
-// Shared-memory shape: rows of RP values, planes of NQ rows.
-template <int NQ>
-struct BoxTile {
-  static constexpr int RP = NQ | 1;        // row, padded to an odd length
-  static constexpr int PP = NQ * RP;       // plane
-  // distance of the tiles of two vector groups when B of them share a CTA,
-  // values of `bytes` bytes: the U values that one 128-byte wavefront serves
-  // come from B groups x U / B lines, so groups lie U / B (mod U) apart
-  static __host__ __device__ constexpr int pitch(int B, int bytes) {
-    const int U = 128 / bytes, want = B >= U ? 1 : U / B, size = NQ * PP;
-    return size + ((want - size) % U + U) % U;
-  }
-};
-
-// A cell along one direction: only its first and last nodes can be shared,
-// wrapped or constrained.
-struct BoxDir {
-  int g0, gP;                    // global coordinates of its nodes 0 and P
-  bool con0, conP, first0, firstP;
-  __device__ __forceinline__ BoxDir(int c, int n, int N, int P, int periodic, int last_odd)
-      : g0(c * P), gP(node_coord(c, P, P, N, periodic)), con0(!periodic && c == 0), conP(!periodic && c == n - 1),
-        first0(first_along(c, n, 0, P, periodic, last_odd)), firstP(first_along(c, n, P, P, periodic, last_odd)) {}
-  __device__ __forceinline__ int at(int i, int P) const { return i == P ? gP : g0 + i; }
-  __device__ __forceinline__ bool con(int i, int P) const { return (i == 0 && con0) || (i == P && conP); }
-  __device__ __forceinline__ bool first(int i, int P) const { return (i != 0 || first0) && (i != P || firstP); }
-};
-
-// N consecutive coefficients, as wide as their alignment (rows of N from an
-// aligned base) allows.
-template <typename G, int N>
-__device__ __forceinline__ void load_row(const G* __restrict__ p, G* c) {
-  constexpr int VW = sizeof(G) == 4 && N % 4 == 0 ? 4 : N % 2 == 0 ? 2 : 1;
-#pragma unroll
-  for (int k = 0; k < N; k += VW) {
-    const Pack<G, VW> v = *reinterpret_cast<const Pack<G, VW>*>(p + k);
-#pragma unroll
-    for (int j = 0; j < VW; ++j) c[k + j] = v.a[j];
-  }
-}
-
 // One cell e and B groups of W vectors: thread (v, ty) of B x nty threads
-// works on group vb B + v.  Switches as in cell_body_eo: SC the scaled
+// works on group vb B + v.  Switches: SC the scaled
 // product, MAP the explicit map of refined meshes, LOCAL the per-cell scratch.
 // vec: X, Y and n_vec are multiples of W values (set by the launch), so a
 // group moves in one access.
@@ -173,7 +70,6 @@ __device__ __forceinline__ void cell_body_box(const BoxTables<typename Arith<V>:
   using D = typename A::D;
   using TS = BoxTile<NQ>;
   constexpr int P = NP - 1, RP = TS::RP, PP = TS::PP, W = A::W;
-  using PK = Pack<D, W>;
   constexpr int HQ = (NQ + 1) / 2, OQ = NQ / 2 > 0 ? NQ / 2 : 1, HP = (NP + 1) / 2, OP = NP / 2 > 0 ? NP / 2 : 1;
   const int pitch = TS::pitch(B, (int)sizeof(V));
   V* T = smem + v * pitch;
@@ -188,32 +84,7 @@ __device__ __forceinline__ void cell_body_box(const BoxTables<typename Arith<V>:
   for (int l = ty; l < NP * NP; l += nty) {
     const int i2 = l % NP, i3 = l / NP;
     V u[NP], a[NQ], ue[HP], uo[OP];
-    if constexpr (MAP) {
-#pragma unroll
-      for (int i1 = 0; i1 < NP; ++i1) {
-        const int code = __ldg(map + (size_t)e * NP * NP * NP + l * NP + i1);
-        const bool use = have > 0 && (code & kMapConstrained) == 0;
-        u[i1] = use ? A::from(load_pack<D, W>(X + (size_t)(code & kMapIndex) * n_vec + vg, have, vec)) : A::zero();
-      }
-    } else {
-      const bool use = have > 0 && !dy.con(i2, P) && !dz.con(i3, P);
-      const size_t row = (dy.at(i2, P) + (size_t)m.Ny * dz.at(i3, P)) * m.Nx;
-#pragma unroll
-      for (int i1 = 0; i1 < NP; ++i1) {
-        const size_t node = row + dx.at(i1, P);
-        if (use && !dx.con(i1, P)) {
-          PK x = load_pack<D, W>(X + node * n_vec + vg, have, vec);
-          if constexpr (SC) {
-            const D ms = __ldg(sc.msq + node);
-#pragma unroll
-            for (int k = 0; k < W; ++k) x.a[k] *= ms;
-          }
-          u[i1] = A::from(x);
-        } else {
-          u[i1] = A::zero();
-        }
-      }
-    }
+    gather_line<A, NP, SC>(node_line<A, NP, 0, MAP>(m, dx, dy, dz, i2, i3, e, map), X, n_vec, vg, have, vec, sc, u);
     eo_split<A, NP>(u, ue, uo);
     eo_parts<A, NQ, NP>(tab.N, ue, uo, a);
     V* dst = T + i3 * PP + i2 * RP;
@@ -315,34 +186,9 @@ __device__ __forceinline__ void cell_body_box(const BoxTables<typename Arith<V>:
   if (have <= 0) return;
   for (int l = ty; l < NP * NP; l += nty) {
     const int i1 = l % NP, i2 = l / NP;
-    // nodes of the line; the values that a later colour adds to are read
-    // before the contraction, and all of them before the first store
-    size_t node[NP];
-    bool con[NP], first[NP];
-    PK old[NP];
-    if constexpr (MAP) {
-#pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        const int code = __ldg(map + (size_t)e * NP * NP * NP + (i * NP + i2) * NP + i1);
-        node[i] = (size_t)(code & kMapIndex);
-        con[i] = (code & kMapConstrained) != 0;
-        first[i] = (code & kMapFirst) != 0;
-      }
-    } else if constexpr (!LOCAL) {
-      const size_t col = dx.at(i1, P) + (size_t)m.Nx * dy.at(i2, P), plane = (size_t)m.Nx * m.Ny;
-      const bool con_xy = dx.con(i1, P) || dy.con(i2, P), first_xy = dx.first(i1, P) && dy.first(i2, P);
-#pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        node[i] = col + plane * dz.at(i, P);
-        con[i] = con_xy || dz.con(i, P);
-        first[i] = first_xy && dz.first(i, P);
-      }
-    }
-    if constexpr (!LOCAL) {
-#pragma unroll
-      for (int i = 0; i < NP; ++i)
-        if (!con[i] && (!first[i] || (SC && sc.c != D(0)))) old[i] = load_pack<D, W>(Y + node[i] * n_vec + vg, have, vec);
-    }
+    const NodeLine<A, NP> nodes = node_line<A, NP, 2, MAP>(m, dx, dy, dz, i1, i2, e, map);
+    Pack<D, W> old[NP];
+    if constexpr (!LOCAL) read_old<A, NP, SC>(nodes, Y, n_vec, vg, have, vec, sc, old);
     V h[NQ], he[HQ], ho[OQ], o[NP];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) h[q] = T[q * PP + i2 * RP + i1];
@@ -354,42 +200,9 @@ __device__ __forceinline__ void cell_body_box(const BoxTables<typename Arith<V>:
 #pragma unroll
       for (int i = 0; i < NP; ++i) store_pack<D, W>(w + (size_t)i * NP * NP * n_vec, A::to(o[i]), have, vec);
     } else {
-#pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        PK r = A::to(o[i]);
-        if constexpr (SC) {
-          // first writer: a M^-1/2 (cell sum) + b X + c Y_old; later ones add
-          const D ams = sc.a * __ldg(sc.msq + node[i]);
-          PK x;
-          if (first[i] && !con[i] && sc.b != D(0)) x = load_pack<D, W>(X + node[i] * n_vec + vg, have, vec);
-#pragma unroll
-          for (int k = 0; k < W; ++k) {
-            r.a[k] *= ams;
-            if (first[i] && !con[i] && sc.b != D(0)) r.a[k] += sc.b * x.a[k];
-            if (first[i] && !con[i] && sc.c != D(0)) r.a[k] += sc.c * old[i].a[k];
-          }
-        }
-        if (first[i]) {
-          if (con[i]) {
-#pragma unroll
-            for (int k = 0; k < W; ++k) r.a[k] = D(0);
-          }
-          store_pack<D, W>(Y + node[i] * n_vec + vg, r, have, vec);
-        } else if (!con[i]) {
-#pragma unroll
-          for (int k = 0; k < W; ++k) r.a[k] = old[i].a[k] + r.a[k];
-          store_pack<D, W>(Y + node[i] * n_vec + vg, r, have, vec);
-        }
-      }
+      scatter_line<A, NP, SC>(nodes, o, old, X, Y, n_vec, vg, have, vec, sc);
     }
   }
-}
-
-// Whether a group of W vectors of X and Y can move in one access.
-template <typename V>
-__host__ __device__ inline bool vec_ok(const void* X, const void* Y, int n_vec) {
-  constexpr size_t bytes = sizeof(typename Arith<V>::D) * Arith<V>::W;
-  return n_vec % Arith<V>::W == 0 && reinterpret_cast<size_t>(X) % bytes == 0 && reinterpret_cast<size_t>(Y) % bytes == 0;
 }
 
 template <typename V, int NP, int NQ, bool SC, bool MAP>
@@ -443,32 +256,6 @@ BoxTables<C, NP, NQ> make_boxtables(const fe_ctx* c) {
   return t;
 }
 
-// Lanes (vector groups) x lines of a CTA, and its shared memory: the tile set
-// with fe_set_tile, or (want.vb = 0) the default one, whose threads a narrow
-// block keeps by taking more lines.
-struct BoxShape {
-  int lanes, lines;
-  size_t smem;
-};
-
-template <typename V, int NQ>
-BoxShape box_shape(LineTile want, int n_vec) {
-  constexpr int W = Arith<V>::W;
-  const LineTile t = want.vb > 0 ? want : Arith<V>::box_tile(NQ);
-  const int groups = (n_vec + W - 1) / W;
-  int b = 1;
-  while (b * 2 * W <= t.vb) b *= 2;
-  const int lanes0 = b;
-  auto bytes = [](int k) { return (size_t)2 * k * BoxTile<NQ>::pitch(k, sizeof(V)) * sizeof(V); };
-  while (b > 1 && bytes(b) > 200 * 1024) b /= 2;
-  while (b > 1 && b / 2 >= groups) b /= 2;
-  int lines = t.lines;
-  if (want.vb <= 0 && b < lanes0) lines = std::min(lines * (lanes0 / b), NQ * NQ);
-  if (b * lines > 256) lines = 256 / b;
-  while ((b * lines) % 32 != 0 && b * lines < 256) ++lines;
-  return BoxShape{b, lines, bytes(b)};
-}
-
 template <typename V, int NP, int NQ, bool SC = false, bool MAP = false>
 cudaError_t launch_box(const fe_ctx* c, const typename Arith<V>::D* X, typename Arith<V>::D* Y, int n_vec,
                        cudaStream_t s, LineTile want, const Geom<typename Arith<V>::G>& geo,
@@ -498,7 +285,7 @@ cudaError_t launch_box(const fe_ctx* c, const typename Arith<V>::D* X, typename 
     }
   }
   auto kern = cell_apply_box_kernel<V, NP, NQ, SC, MAP>;
-  const BoxShape sh = box_shape<V, NQ>(want, n_vec);
+  const BoxShape sh = box_shape<V, NQ, 2>(want, Arith<V>::box_tile(NQ), n_vec);
   cudaError_t e = ensure_dyn_smem(reinterpret_cast<const void*>(kern), sh.smem);
   if (e != cudaSuccess) return e;
   const int n_vb = (n_vec + sh.lanes * W - 1) / (sh.lanes * W);

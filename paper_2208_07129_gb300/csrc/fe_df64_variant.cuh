@@ -5,7 +5,7 @@
 #pragma once
 
 #include "fe_box.cuh"
-#include "fe_ff_body.cuh"
+#include "fe_general.cuh"
 
 namespace fe {
 
@@ -14,7 +14,7 @@ cudaError_t apply_df64_variant(const fe_ctx* c, const double* X, double* Y, int 
                                const Scale<double>& sc) {
 #define FE_CASE(P, NQ) \
   if (c->p == P && c->nq == NQ) {                                                                     \
-    if constexpr (GEN) return launch_df64<P + 1, NQ, SC>(c, X, Y, n_vec, s, sc);                       \
+    if constexpr (GEN) return launch_general<ff, P + 1, NQ, SC>(c, X, Y, n_vec, s, c->tiledf(), make_geom<ff>(c), sc); \
     else return launch_box<ff, P + 1, NQ, SC>(c, X, Y, n_vec, s, c->tiledf(), make_geom<ff>(c), sc); \
   }
   FE_FOR_EACH_P_NQ(FE_CASE)

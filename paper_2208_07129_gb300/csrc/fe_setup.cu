@@ -319,10 +319,9 @@ extern "C" fe_status fe_setup(const fe_mesh_desc* mesh, int p, const fe_quad_des
   c->periodic = mesh->bc == FE_BC_PERIODIC;
   c->p = p; c->np = p + 1; c->nq = quad->n_q; c->quad_kind = quad->kind; c->mu = mu;
   c->general = mesh->vertex_xyz != nullptr;
-  // FP64 tile measured on GB300: 8 vectors x 16 lines up to n_q = 8, 4 x 32 above;
-  // FP32: even-odd line kernel, 8 x 32 up to n_q = 8, 4 x 64 above (two more
-  // CTAs per SM in the 48 KB of shared memory that 4 vectors of n_q = 10 take)
-  // double-float: 8 x 32 up to n_q = 8, 4 x 64 above
+  // tiles of the plain line kernels (variant 1), measured on GB300: FP64 8
+  // vectors x 16 lines up to n_q = 8, 4 x 32 above; FP32 8 x 32 and 4 x 64.  The
+  // default kernels have their own (Arith::box_tile, Arith::general_tile).
   c->fp32_variant = 3;
   if (quad->n_q >= 9) { c->vb64 = 4; c->nty64 = 32; c->vb32 = 4; c->nty32 = 64; c->vbdf = 4; c->ntydf = 64; }
   const int np = c->np, nq = c->nq;
