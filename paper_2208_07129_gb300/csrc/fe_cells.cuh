@@ -113,19 +113,6 @@ struct BoxTile {
   }
 };
 
-// A cell along one direction: only its first and last nodes can be shared,
-// wrapped or constrained.
-struct BoxDir {
-  int g0, gP;                    // global coordinates of its nodes 0 and P
-  bool con0, conP, first0, firstP;
-  __device__ __forceinline__ BoxDir(int c, int n, int N, int P, int periodic, int last_odd)
-      : g0(c * P), gP(node_coord(c, P, P, N, periodic)), con0(!periodic && c == 0), conP(!periodic && c == n - 1),
-        first0(first_along(c, n, 0, P, periodic, last_odd)), firstP(first_along(c, n, P, P, periodic, last_odd)) {}
-  __device__ __forceinline__ int at(int i, int P) const { return i == P ? gP : g0 + i; }
-  __device__ __forceinline__ bool con(int i, int P) const { return (i == 0 && con0) || (i == P && conP); }
-  __device__ __forceinline__ bool first(int i, int P) const { return (i != 0 || first0) && (i != P || firstP); }
-};
-
 // N consecutive coefficients, as wide as their alignment (rows of N from an
 // aligned base) allows.
 template <typename G, int N>

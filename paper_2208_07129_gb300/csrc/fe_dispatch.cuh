@@ -35,6 +35,22 @@ cudaError_t launch_kernel(void (*kern)(P...), size_t blocks, dim3 threads, size_
   return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 
+// A cell along one direction: only its first and last nodes can be shared,
+// wrapped or constrained.
+struct BoxDir {
+  int g0, gP;                    // global coordinates of its nodes 0 and P
+  bool con0, conP, first0, firstP, shared0, sharedP;
+  __device__ __forceinline__ BoxDir(int c, int n, int N, int P, int periodic, int last_odd)
+      : g0(c * P), gP(node_coord(c, P, P, N, periodic)), con0(!periodic && c == 0), conP(!periodic && c == n - 1),
+        first0(first_along(c, n, 0, P, periodic, last_odd)), firstP(first_along(c, n, P, P, periodic, last_odd)),
+        shared0(c > 0 || periodic), sharedP(c < n - 1 || periodic) {}
+  __device__ __forceinline__ int at(int i, int P) const { return i == P ? gP : g0 + i; }
+  __device__ __forceinline__ bool con(int i, int P) const { return (i == 0 && con0) || (i == P && conP); }
+  __device__ __forceinline__ bool first(int i, int P) const { return (i != 0 || first0) && (i != P || firstP); }
+  // whether a second cell of the direction holds the node
+  __device__ __forceinline__ bool shared(int i, int P) const { return (i == 0 && shared0) || (i == P && sharedP); }
+};
+
 template <typename T, int NP, int NQ>
 Tables<T, NP, NQ> make_tables(const fe_ctx* c) {
   Tables<T, NP, NQ> t;

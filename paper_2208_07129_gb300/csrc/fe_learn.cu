@@ -16,12 +16,12 @@
 // has no learned component; this layer sits on top of its operator.
 //
 // Kernels:
-//  * inference: one fused kernel per cell colour.  A CTA takes one cell and
-//    128 columns (patches): it gathers the 128 x n_p^3 patch tile into shared
-//    memory as BF16, runs GEMM1 (128 x 128 x K1) and GEMM2 (128 x K1 x 128) on
-//    the 5th-generation tensor cores (tcgen05.mma kind::f16, BF16 operands,
-//    FP32 accumulators in tensor memory), applies 1/s, b1 and ReLU between
-//    them, and scales and assembles the output into z.  Colours make the
+//  * inference: one fused persistent kernel per cell colour.  A task is one cell
+//    and 128 columns (patches): the 128 x n_p^3 patch tile is gathered into
+//    tensor memory as BF16, GEMM1 (128 x 128 x K1) and GEMM2 (128 x K1 x 128)
+//    run on the 5th-generation tensor cores (tcgen05.mma kind::f16, BF16
+//    operands, FP32 accumulators in tensor memory), 1/s, b1 and ReLU are
+//    applied between them, and the output is scaled and assembled into z.  Colours make the
 //    assembly conflict-free, as in the operator.
 //  * training: FP32 CUDA-core GEMMs (strided, tiled) for forward and backward,
 //    column-sum bias gradients, and Adam, all on the device.
@@ -36,7 +36,7 @@
 #include <cuda_bf16.h>
 
 #include "fe_internal.h"
-#include "fe_cell_kernel.cuh"
+#include "fe_dispatch.cuh"
 #include "fe_umma.cuh"
 #include "../../include/fe_learn.h"
 
@@ -84,181 +84,301 @@ struct MlpArgs {
   int n3, K1, np;
 };
 
-// z += sum over this colour's cells of R_e^T (w .* s MLP(R_e r / s)) for 128
-// columns per CTA.  256 threads: thread t serves column (row of the tile)
-// t % 128 and half t / 128 of the work of that row (alternate node chunks in
-// the gather, alternate 32-column groups in the epilogues), so twice as many
-// loads and stores are in flight; warp w reads the TMEM lanes of its quarter
-// w % 4.
-constexpr int kMlpThreads = 256;
+// z = D^-1 r + sum over the cells of R_e^T (w .* s MLP(R_e r / s)), the cells of
+// one colour per launch: the first colour of a node stores D^-1 r plus its
+// share, later ones add theirs.
+//
+// Persistent: one CTA per SM takes tasks (a cell x 128 columns) in turn, with
+// both weight images resident in shared memory (2 x 88 KB at p = 6).  The A
+// operands live in tensor memory (lane = column of the block, two BF16 of
+// consecutive K per 32-bit word): the patch (K1 / 2 words), the hidden layer
+// (64) and two 128-word accumulators fit its 512 words, so shared memory holds
+// no tile and the gather of the next task overlaps the epilogue of this one:
+//   warps 0-7   gather: thread = column x half of the node chunks; FP32 loads,
+//               BF16 pairs to tensor memory, sum of squares; GEMM1
+//   warps 8-15  hidden layer (1/s, b1, ReLU), GEMM2 in chunks of 128 outputs
+//               alternating between the accumulators, scatter
+// What bounds it: the issue of the gather's and scatter's 128-byte loads (a
+// warp's 32 independent loads take 4-7 K cycles to issue, the wait for their
+// data 1 K more); the tensor pipe is idle.  One application on 24^3 cells, p =
+// 6, 128 columns: 6.37 -> 3.18 ms (24^3, p = 4, 100 columns 2.28 -> 1.25 ms)
+// against a kernel that reloaded both images into one 218 KB CTA per task, with
+// gather, GEMMs and scatter taking turns and z initialised in a pass of its own.
+constexpr int kMlpThreads = 512;
+constexpr int kMlpHalf = 256;                       // threads of each role
+constexpr uint32_t kTmPatch = 0, kTmAcc0 = 176, kTmHidden = 304, kTmAcc1 = 368;   // tensor-memory words
+
+// A named barrier of `count` threads that also tells whether `ok` held for all.
+__device__ __forceinline__ bool barrier_and(int id, int count, bool ok) {
+  int r;
+  asm volatile(
+      "{\n.reg .pred p, q;\nsetp.ne.s32 p, %1, 0;\nbarrier.cta.red.and.pred q, %2, %3, p;\nselp.s32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"((int)ok), "r"(id), "r"(count)
+      : "memory");
+  return r != 0;
+}
+
+// 4 / 16 words of this thread's tensor-memory lane.
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, uint4 v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr), "r"(v.x), "r"(v.y), "r"(v.z),
+               "r"(v.w)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// D[tmem] (+)= A[tmem] . B[smem]^T, issued by one thread.
+__device__ __forceinline__ void umma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t idesc,
+                                             uint32_t acc) {
+  asm volatile(
+      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(b), "r"(idesc), "r"(acc));
+}
+
+// A node of a task's cell.
+struct alignas(16) MlpNode {
+  long long code;   // 4 DoF + 1 (constrained) + 2 (its first colour), -1 past the patch
+  float w, d;       // partition-of-unity weight; 1 / D for a first colour, else 1
+};
+
+struct MlpShared {
+  unsigned char *w1, *w2;
+  MlpNode* node;     // [2][K1]
+  float* b2;         // [K1]
+  float* ssq;        // [2][2][128]: partial squared norms
+  uint64_t* bar;     // GEMM1 done, GEMM2 chunks 0..2 done, task's accumulators read
+  uint32_t* tslot;
+};
+
+__host__ __device__ constexpr size_t mlp_smem_bytes(int K1) {
+  return (size_t)2 * kTile * K1 * 2 + (size_t)K1 * (2 * sizeof(MlpNode) + 4) + 4 * kTile * sizeof(float) + 6 * 8 + 16;
+}
+
 __global__ void __launch_bounds__(kMlpThreads, 1) mlp_precond_kernel(const MlpArgs a, const MeshDev m,
-                                                                     const int* __restrict__ cells,
+                                                                     const int* __restrict__ cells, int n_tasks,
                                                                      const float* __restrict__ R,
-                                                                     float* __restrict__ Z, int n_vec, int n_cb,
-                                                                     int* status) {
+                                                                     const float* __restrict__ dinv, float* Z,
+                                                                     int n_vec, int n_cb, int* status) {
   extern __shared__ __align__(1024) unsigned char smem[];
-  const size_t img = (size_t)kTile * a.K1 * 2;
-  unsigned char* reg0 = smem;             // patch tile, then W2 image
-  unsigned char* reg1 = smem + img;       // W1 image
-  unsigned char* reg2 = reg1 + img;       // hidden tile (128 x 128 BF16)
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(reg2 + kTile * kHidden * 2);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 1);
-  float* ssq = reinterpret_cast<float*>(tslot + 4);   // [2][128] partial squared norms
-  long long* noff = reinterpret_cast<long long*>(ssq + 2 * kTile);   // per node: global DoF, -1 if constrained
-  float* nw = reinterpret_cast<float*>(noff + a.K1);                // per node: partition-of-unity weight
+  const int K1 = a.K1;
+  const size_t img = (size_t)kTile * K1 * 2;
+  MlpShared sh;
+  sh.w1 = smem;
+  sh.w2 = smem + img;
+  sh.node = reinterpret_cast<MlpNode*>(smem + 2 * img);
+  sh.b2 = reinterpret_cast<float*>(sh.node + 2 * K1);
+  sh.bar = reinterpret_cast<uint64_t*>(sh.b2 + K1);
+  sh.ssq = reinterpret_cast<float*>(sh.bar + 6);
+  sh.tslot = reinterpret_cast<uint32_t*>(sh.ssq + 4 * kTile);
+  uint64_t *bar_g1 = sh.bar, *bar_g2 = sh.bar + 1, *bar_read = sh.bar + 4;
 
   const int t = threadIdx.x, warp = t >> 5;
-  const int row = t & (kTile - 1), half = t >> 7;
-  const int cb = blockIdx.x % n_cb;
-  const int e = cells[blockIdx.x / n_cb];
-  const int col = cb * kTile + row;
-  const bool active = col < n_vec;
+  const int row = t & (kTile - 1), half = (t >> 7) & 1;
+  const int n_chunks = (K1 + 127) / 128;
   const int P = a.np - 1;
-  const int cx = e % m.nx, cy = (e / m.nx) % m.ny, cz = e / (m.nx * m.ny);
 
+  let_next_launch_start();
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(sh.tslot)),
                  "r"(kTmemCols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
-  if (t == 0) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(mbar)));
-
-  // the cell's node offsets and weights, once per CTA
-  for (int i = t; i < a.K1; i += kMlpThreads) {
-    long long off = -1;
-    float wgt = 0.f;
-    if (i < a.n3) {
-      size_t dof;
-      bool con;
-      node_info(m, P, a.np, cx, cy, cz, i, &dof, &con, &wgt);
-      off = con ? -1 : (long long)dof;
-    }
-    noff[i] = off;
-    nw[i] = wgt;
-  }
-  // W1 image -> shared (straight 16-byte copy)
-  {
-    const uint4* src = reinterpret_cast<const uint4*>(a.W1img);
-    uint4* dst = reinterpret_cast<uint4*>(reg1);
-#pragma unroll 4
-    for (size_t k = t; k < img / 16; k += kMlpThreads) dst[k] = __ldg(src + k);
-  }
-  __syncthreads();
-  // gather the patch of column `col` (row `row` of the tile), 8 nodes per 16-byte chunk
-  float ss = 0.f;
-#pragma unroll 4
-  for (int kg = half; kg < a.K1 / 8; kg += 2) {
-    float v[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const long long off = noff[kg * 8 + u];
-      v[u] = (active && off >= 0) ? __ldg(R + off * n_vec + col) : 0.f;
-    }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) ss += v[u] * v[u];
-    uint4 chunk;
-    chunk.x = pack_bf16(v[0], v[1]);
-    chunk.y = pack_bf16(v[2], v[3]);
-    chunk.z = pack_bf16(v[4], v[5]);
-    chunk.w = pack_bf16(v[6], v[7]);
-    *reinterpret_cast<uint4*>(reg0 + core_offset(row, kg * 8, a.K1)) = chunk;
-  }
-  ssq[half * kTile + row] = ss;
-
-  asm volatile("fence.proxy.async.shared::cta;");
-  asm volatile("fence.mbarrier_init.release.cluster;");
-  asm volatile("tcgen05.fence::before_thread_sync;");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  const uint32_t tmem = *tslot;
-  const float s2 = ssq[row] + ssq[kTile + row];
-  const float s = sqrtf(s2);
-  const float inv_s = s2 > 0.f ? 1.0f / s : 0.f;
-  const uint32_t sbo1 = (uint32_t)(a.K1 / 8) * 128;
-
-  // GEMM1: D1[128 patches x 128 hidden] = tile[128 x K1] . W1^T
   if (t == 0) {
-    const uint32_t idesc = umma_idesc_bf16(kTile, kHidden);
-    for (int k = 0; k < a.K1 / 16; ++k)
-      umma_bf16(tmem, umma_desc(smem_u32(reg0) + k * 256, 128, sbo1), umma_desc(smem_u32(reg1) + k * 256, 128, sbo1),
-                idesc, k > 0);
-    umma_commit(mbar);
+    for (int k = 0; k < 5; ++k) mbar_init(sh.bar + k, k == 0 ? 2 : 1);
+    asm volatile("fence.mbarrier_init.release.cluster;");
   }
-  bool ok = mbar_wait_timed(mbar, 0);
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  // every thread must see GEMM1 complete before the patch tile is overwritten
-  __syncthreads();
-  const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-  if (ok) {
-    // the patch tile is consumed: bring the W2 image into its place
-    const uint4* src = reinterpret_cast<const uint4*>(a.W2img);
-    uint4* dst = reinterpret_cast<uint4*>(reg0);
+  for (int i = 0; i < 2; ++i) {   // both images, straight 16-byte copies
+    const uint4* src = reinterpret_cast<const uint4*>(i ? a.W2img : a.W1img);
+    uint4* dst = reinterpret_cast<uint4*>(i ? sh.w2 : sh.w1);
 #pragma unroll 4
     for (size_t k = t; k < img / 16; k += kMlpThreads) dst[k] = __ldg(src + k);
-    // h = relu(D1 / s + b1) -> BF16 hidden tile, row `row`, columns of this half
-    for (int c0 = half * 32; c0 < kHidden; c0 += 64) {
-      float d[32];
-      tmem_ld32(lane_base + c0, d);
+  }
+  for (int i = t; i < K1; i += kMlpThreads) sh.b2[i] = i < a.n3 ? __ldg(a.b2 + i) : 0.f;
+  fence_async_smem();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *sh.tslot;
+  const uint32_t lane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+  bool ok = true;
+
+  if (t < kMlpHalf) {
+    // ---- gather, GEMM1 ----
+    // local node of each of this thread's table entries (at most two: K1 <= 512)
+    int li[2][3];
 #pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        float h[8];
+    for (int r = 0; r < 2; ++r) {
+      const int i = t + r * kMlpHalf;
+      li[r][0] = i % a.np;
+      li[r][1] = (i / a.np) % a.np;
+      li[r][2] = i / (a.np * a.np);
+    }
+    int it = 0, e_next = __ldg(cells + min((int)blockIdx.x, n_tasks - 1) / n_cb);
+    for (int task = blockIdx.x; task < n_tasks; task += gridDim.x, ++it) {
+      const int buf = it & 1;
+      const int e = e_next;
+      e_next = __ldg(cells + min(task + (int)gridDim.x, n_tasks - 1) / n_cb);
+      // the task's nodes (this buffer's last user is the scatter of task
+      // it - 2, done before GEMM1 of task it - 1 was issued)
+      const BoxDir dx(e % m.nx, m.nx, m.Nx, P, m.periodic, m.last_odd_x);
+      const BoxDir dy((e / m.nx) % m.ny, m.ny, m.Ny, P, m.periodic, m.last_odd_y);
+      const BoxDir dz(e / (m.nx * m.ny), m.nz, m.Nz, P, m.periodic, m.last_odd_z);
+      MlpNode rec[2];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) h[u] = fmaxf(fmaf(d[g * 8 + u], inv_s, __ldg(a.b1 + c0 + g * 8 + u)), 0.f);
-        uint4 chunk;
-        chunk.x = pack_bf16(h[0], h[1]);
-        chunk.y = pack_bf16(h[2], h[3]);
-        chunk.z = pack_bf16(h[4], h[5]);
-        chunk.w = pack_bf16(h[6], h[7]);
-        *reinterpret_cast<uint4*>(reg2 + core_offset(row, c0 + g * 8, kHidden)) = chunk;
+      for (int r = 0; r < 2; ++r) {
+        rec[r] = MlpNode{-1, 0.f, 1.f};
+        if (t + r * kMlpHalf < a.n3) {
+          const int i1 = li[r][0], i2 = li[r][1], i3 = li[r][2];
+          const size_t dof = dx.at(i1, P) + (size_t)m.Nx * (dy.at(i2, P) + (size_t)m.Ny * dz.at(i3, P));
+          const bool con = dx.con(i1, P) || dy.con(i2, P) || dz.con(i3, P);
+          const bool first = dx.first(i1, P) && dy.first(i2, P) && dz.first(i3, P);
+          const int shared = (dx.shared(i1, P) ? 2 : 1) * (dy.shared(i2, P) ? 2 : 1) * (dz.shared(i3, P) ? 2 : 1);
+          rec[r].code = 4 * (long long)dof + (con ? 1 : 0) + (first ? 2 : 0);
+          rec[r].w = 1.0f / (float)shared;
+          if (first) rec[r].d = __ldg(dinv + dof);
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+        if (t + r * kMlpHalf < K1) sh.node[buf * K1 + t + r * kMlpHalf] = rec[r];
+      ok = barrier_and(1, kMlpHalf, ok);
+      if (!ok) break;
+      const int col = (task % n_cb) * kTile + row;
+      const bool active = col < n_vec;
+      const MlpNode* node = sh.node + buf * K1;
+      float ss = 0.f;
+      // 8-node chunks kg = half, half + 2, ...; four chunks' loads at once
+      for (int k0 = half; k0 < K1 / 8; k0 += 8) {
+        float v[4][8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const int i = (k0 + 2 * j) * 8 + u;
+            v[j][u] = 0.f;
+            const long long nd = i < K1 ? node[i].code : -1;
+            if (active && nd >= 0 && !(nd & 1)) v[j][u] = __ldg(R + (nd >> 2) * n_vec + col);
+          }
+        // the patch of task it - 1 is read once its GEMM1 is done
+        if (k0 == half && it > 0) ok = __all_sync(~0u, mbar_wait_timed(bar_g1, (it - 1) & 1));
+        tc_fence_after();
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (k0 + 2 * j >= K1 / 8) continue;
+#pragma unroll
+          for (int u = 0; u < 8; ++u) ss += v[j][u] * v[j][u];
+          tmem_st4(lane + kTmPatch + (k0 + 2 * j) * 4,
+                   make_uint4(pack_bf16(v[j][0], v[j][1]), pack_bf16(v[j][2], v[j][3]), pack_bf16(v[j][4], v[j][5]),
+                              pack_bf16(v[j][6], v[j][7])));
+        }
+      }
+      sh.ssq[(buf * 2 + half) * kTile + row] = ss;
+      tmem_wait_st();
+      // GEMM1 writes accumulator 0: the scatter of task it - 1 has to be done
+      if (t == 0 && it > 0) ok = ok && mbar_wait_timed(bar_read, (it - 1) & 1);
+      tc_fence_before();
+      ok = barrier_and(1, kMlpHalf, ok);
+      if (!ok) break;
+      if (t == 0) {
+        tc_fence_after();
+        const uint32_t idesc = umma_idesc_bf16(kTile, kHidden), sbo1 = (uint32_t)(K1 / 8) * 128;
+        for (int k = 0; k < K1 / 16; ++k)
+          umma_bf16_ta(tmem + kTmAcc0, tmem + kTmPatch + k * 8, umma_desc(smem_u32(sh.w1) + k * 256, 128, sbo1), idesc,
+                       k > 0);
+        umma_commit(bar_g1);
+        // the second arrival publishes the gather's tables and norms
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar_g1)) : "memory");
       }
     }
-  } else if (t == 0) {
-    atomicMax(status, (int)FE_ETIMEOUT);
-  }
-  asm volatile("fence.proxy.async.shared::cta;");
-  asm volatile("tcgen05.fence::before_thread_sync;");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;");
-
-  // GEMM2: D2[128 x K1] = hidden[128 x 128] . W2^T, in N chunks of <= 256
-  if (ok && t == 0) {
+  } else {
+    // ---- hidden layer, GEMM2, scatter ----
     const uint32_t sbo2 = (uint32_t)(kHidden / 8) * 128;
-    for (int n0 = 0; n0 < a.K1; n0 += 256) {
-      const int nn = a.K1 - n0 < 256 ? a.K1 - n0 : 256;
+    auto issue_chunk = [&](int j) {   // one thread
+      const int n0 = 128 * j, nn = K1 - n0 < 128 ? K1 - n0 : 128;
       const uint32_t idesc = umma_idesc_bf16(kTile, nn);
       for (int k = 0; k < kHidden / 16; ++k)
-        umma_bf16(tmem + kHidden + n0, umma_desc(smem_u32(reg2) + k * 256, 128, sbo2),
-                  umma_desc(smem_u32(reg0) + (uint32_t)(n0 / 8) * sbo2 + k * 256, 128, sbo2), idesc, k > 0);
-    }
-    umma_commit(mbar);
-  }
-  if (ok) ok = mbar_wait_timed(mbar, 1);
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  if (ok) {
-    for (int c0 = half * 32; c0 < a.K1; c0 += 64) {
-      float d[32];
-      tmem_ld32(lane_base + kHidden + c0, d);
-      if (!active) continue;
-      // all 32 reads of z are issued before the first store (a store may
-      // alias a later read as far as the compiler knows), so they overlap
-      float zold[32];
+        umma_bf16_ta(tmem + (j & 1 ? kTmAcc1 : kTmAcc0), tmem + kTmHidden + k * 8,
+                     umma_desc(smem_u32(sh.w2) + (uint32_t)(n0 / 8) * sbo2 + k * 256, 128, sbo2), idesc, k > 0);
+      umma_commit(bar_g2 + j);
+    };
+    int it = 0;
+    for (int task = blockIdx.x; task < n_tasks; task += gridDim.x, ++it) {
+      const int buf = it & 1;
+      const int col = (task % n_cb) * kTile + row;
+      const bool active = col < n_vec;
+      ok = __all_sync(~0u, mbar_wait_timed(bar_g1, it & 1));
+      tc_fence_after();
+      const float s2 = sh.ssq[buf * 2 * kTile + row] + sh.ssq[(buf * 2 + 1) * kTile + row];
+      const float s = sqrtf(s2);
+      const float inv_s = s2 > 0.f ? 1.0f / s : 0.f;
+      if (ok) {
+        for (int c0 = half * 32; c0 < kHidden; c0 += 64) {   // h = relu(D1 / s + b1) -> BF16
+          float d[32];
+          tmem_ld32(lane + kTmAcc0 + c0, d);
 #pragma unroll
-      for (int u = 0; u < 32; ++u) {
-        const int i = c0 + u;
-        const long long off = i < a.n3 ? noff[i] : -1;
-        zold[u] = off >= 0 ? Z[off * n_vec + col] : 0.f;
-      }
+          for (int g = 0; g < 4; ++g) {
+            float h[8];
 #pragma unroll
-      for (int u = 0; u < 32; ++u) {
-        const int i = c0 + u;
-        const long long off = i < a.n3 ? noff[i] : -1;
-        if (off >= 0) Z[off * n_vec + col] = zold[u] + (d[u] + __ldg(a.b2 + i)) * s * nw[i];
+            for (int u = 0; u < 8; ++u) h[u] = fmaxf(fmaf(d[g * 8 + u], inv_s, __ldg(a.b1 + c0 + g * 8 + u)), 0.f);
+            tmem_st4(lane + kTmHidden + c0 / 2 + g * 4, make_uint4(pack_bf16(h[0], h[1]), pack_bf16(h[2], h[3]),
+                                                                   pack_bf16(h[4], h[5]), pack_bf16(h[6], h[7])));
+          }
+        }
+        tmem_wait_st();
       }
+      tc_fence_before();
+      ok = barrier_and(2, kMlpHalf, ok);
+      if (!ok) break;
+      tc_fence_after();
+      if (t == kMlpHalf) {
+        issue_chunk(0);
+        if (n_chunks > 1) issue_chunk(1);
+      }
+      if (it == 0) wait_for_earlier_launch();   // z of the colours before
+      const MlpNode* node = sh.node + buf * K1;
+      for (int j = 0; j < n_chunks; ++j) {
+        if (ok) ok = mbar_wait_timed(bar_g2 + j, it & 1);
+        ok = __all_sync(~0u, ok);
+        tc_fence_after();
+        const int end = K1 - 128 * j < 128 ? K1 - 128 * j : 128;
+        for (int c0 = half * 32; ok && c0 < end; c0 += 64) {
+          float d[32], zold[32];
+          tmem_ld32(lane + (j & 1 ? kTmAcc1 : kTmAcc0) + c0, d);
+          if (!active) continue;
+          // all 32 reads (r for a first colour, z otherwise) are issued before
+          // anything uses them or the first store
+#pragma unroll
+          for (int u = 0; u < 32; ++u) {
+            const int i = 128 * j + c0 + u;
+            const long long nd = i < K1 ? node[i].code : -1;
+            const float* src = nd & 2 ? R : Z;
+            zold[u] = 0.f;
+            if (nd >= 0 && (nd & 3) != 1) zold[u] = src[(nd >> 2) * n_vec + col];
+          }
+#pragma unroll
+          for (int u = 0; u < 32; ++u) {
+            const int i = 128 * j + c0 + u;
+            const MlpNode nd = node[i < K1 ? i : 0];
+            const float z = __fmul_rn(zold[u], nd.d);   // D^-1 r, or z as it is
+            const float zn = z + (d[u] + sh.b2[i < K1 ? i : 0]) * s * nd.w;
+            if (i < a.n3 && (nd.code & 3) != 1) Z[(nd.code >> 2) * n_vec + col] = nd.code & 1 ? z : zn;
+          }
+        }
+        tc_fence_before();
+        ok = barrier_and(2, kMlpHalf, ok);   // accumulator j & 1 is read
+        if (!ok) break;
+        tc_fence_after();
+        if (t == kMlpHalf && j + 2 < n_chunks) issue_chunk(j + 2);
+      }
+      if (!ok) break;
+      if (t == kMlpHalf)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar_read)) : "memory");
     }
-  } else if (t == 0) {
-    atomicMax(status, (int)FE_ETIMEOUT);
   }
-  asm volatile("tcgen05.fence::before_thread_sync;");
+  if (!ok) atomicMax(status, (int)FE_ETIMEOUT);
+  wait_for_earlier_launch();   // every CTA, so that completion is in colour order
+  tc_fence_before();
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
 }
@@ -702,10 +822,6 @@ static fe_status from_cuda(cudaError_t e) {
   return fe::cuda_status(e);
 }
 
-static size_t smem_bytes(int K1) {
-  return (size_t)2 * kTile * K1 * 2 + kTile * kHidden * 2 + 32 + 2 * kTile * 4 + (size_t)K1 * 12;
-}
-
 static cudaError_t alloc_learned(fe_ctx* c) {
   if (c->learned) return cudaSuccess;
   LearnedPrecond* L = new LearnedPrecond();
@@ -764,19 +880,24 @@ fe_status precond_apply_f32(fe_ctx* c, const float* r, float* z, int nv, cudaStr
   if (L->K1 > 352) return FE_EUNSUPPORTED;
   cudaError_t e = solver_workspace(c, 1);
   if (e != cudaSuccess) return from_cuda(e);
-  const size_t n = c->n_dofs;
-  jacobi_init_kernel<<<grid_for(n * nv), 256, 0, s>>>(r, c->ws.dinv32, z, n, nv);
-  const size_t smem = smem_bytes(L->K1);
+  const size_t smem = mlp_smem_bytes(L->K1);
   e = ensure_dyn_smem(reinterpret_cast<const void*>(mlp_precond_kernel), smem);
+  int dev = 0, sms = 0;
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return from_cuda(e);
   MlpArgs a{L->W1img, L->W2img, L->b1, L->b2, L->n3, L->K1, c->np};
   const int n_cb = (nv + kTile - 1) / kTile;
+  bool overlap = false;
   for (int k = 0; k < c->colors.n_colors; ++k) {
     const int nc = c->colors.offset[k + 1] - c->colors.offset[k];
     if (nc == 0) continue;
-    mlp_precond_kernel<<<(unsigned)((long long)nc * n_cb), kMlpThreads, smem, s>>>(
-        a, c->mdev, c->d_cells + c->colors.offset[k], r, z, nv, n_cb, c->d_status);
-    if ((e = cudaGetLastError()) != cudaSuccess) return from_cuda(e);
+    const long long tasks = (long long)nc * n_cb;
+    if (tasks > 0x7fffffffLL) return from_cuda(cudaErrorInvalidConfiguration);
+    e = launch_kernel(mlp_precond_kernel, (size_t)std::min<long long>(tasks, sms), dim3(kMlpThreads), smem, s, overlap, a,
+                      c->mdev, c->d_cells + c->colors.offset[k], (int)tasks, r, c->ws.dinv32, z, nv, n_cb, c->d_status);
+    if (e != cudaSuccess) return from_cuda(e);
+    overlap = true;
   }
   return FE_OK;
 }
