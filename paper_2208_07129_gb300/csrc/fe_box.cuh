@@ -266,18 +266,18 @@ cudaError_t launch_box(const fe_ctx* c, const typename Arith<V>::D* X, typename 
   const BoxTables<typename Arith<V>::C, NP, NQ> tab = make_boxtables<typename Arith<V>::C, NP, NQ>(c);
   if constexpr (!SC && !MAP) {
     // Small meshes (scratch allocated at setup): one launch over all cells
-    // (one vector group per CTA, so even a few cells fill the GPU) writing
-    // each cell's result to the scratch, then one gather in colour order.
+    // writing each cell's result to the scratch, then one gather in colour order.
     if (c->d_small && (size_t)n_vec * NP * NP * NP * c->n_cells * sizeof(D) <= c->small_bytes) {
       auto lk = cell_apply_box_local_kernel<V, NP, NQ>;
-      constexpr int lines = NQ * NQ < 64 ? 32 : 64;
-      const size_t lsm = (size_t)2 * BoxTile<NQ>::pitch(1, sizeof(V)) * sizeof(V);
-      cudaError_t e = ensure_dyn_smem(reinterpret_cast<const void*>(lk), lsm);
+      int lanes = 1;
+      size_t lsm = 0;
+      cudaError_t e = small_shape<V, NQ, 2>(c->n_cells, n_vec, &lanes, &lsm);
+      if (e == cudaSuccess) e = ensure_dyn_smem(reinterpret_cast<const void*>(lk), lsm);
       if (e != cudaSuccess) return e;
       D* Wk = static_cast<D*>(c->d_small);
-      const int groups = (n_vec + W - 1) / W;
-      e = launch_kernel(lk, c->n_cells * (size_t)groups, dim3(1, lines), lsm, s, false, tab, c->mdev, geo, n_vec, groups,
-                        vec, X, Wk);
+      const int blocks = (n_vec + lanes * W - 1) / (lanes * W);
+      e = launch_kernel(lk, c->n_cells * (size_t)blocks, dim3(lanes, NQ * NQ), lsm, s, false, tab, c->mdev, geo, n_vec,
+                        blocks, vec, X, Wk);
       if (e != cudaSuccess) return e;
       const size_t tot = c->n_dofs * (size_t)n_vec;
       return launch_kernel(assemble_local_kernel<D, NP>, std::min<size_t>((tot + 255) / 256, 152 * 8), dim3(256), 0, s,

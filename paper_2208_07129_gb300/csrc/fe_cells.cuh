@@ -247,6 +247,34 @@ __host__ __device__ inline bool vec_ok(const void* X, const void* Y, int n_vec) 
   return n_vec % Arith<V>::W == 0 && reinterpret_cast<size_t>(X) % bytes == 0 && reinterpret_cast<size_t>(Y) % bytes == 0;
 }
 
+// CTA of a small mesh: every line of a pass has a thread, and B vector groups
+// share a CTA, B chosen so that the fullest SM has the fewest warps: with few
+// cells a CTA's time is its passes' latency, and partly filled warps cost the
+// FP64 pipe as much as full ones (4^3 cells, n_q = 6, 8 vectors: 128 CTAs of 4 x
+// 36 threads put 5 warps on an SM, 512 CTAs of one 36-line vector put 8).
+template <typename V, int NQ, int TILES>
+cudaError_t small_shape(size_t cells, int n_vec, int* lanes, size_t* smem) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const int groups = (n_vec + Arith<V>::W - 1) / Arith<V>::W;
+  size_t best = 0;
+  *lanes = 1;
+  for (int b = 1; b == 1 || (b * NQ * NQ <= 256 && b / 2 < groups); b *= 2) {
+    const size_t bytes = (size_t)TILES * b * BoxTile<NQ>::pitch(b, sizeof(V)) * sizeof(V);
+    if (bytes > 100 * 1024 && b > 1) break;
+    const size_t ctas = cells * ((groups + b - 1) / b);
+    const size_t cost = (ctas + sms - 1) / sms * ((b * NQ * NQ + 31) / 32);
+    if (best == 0 || cost < best) {
+      best = cost;
+      *lanes = b;
+      *smem = bytes;
+    }
+  }
+  return cudaSuccess;
+}
+
 // Lanes (vector groups) x lines of a CTA, and its shared memory: the tile set
 // with fe_set_tile, or (want.vb = 0) the default one, whose threads a narrow
 // block keeps by taking more lines.
