@@ -19,20 +19,26 @@ __device__ __forceinline__ void let_next_launch_start() { asm volatile("griddepc
 __device__ __forceinline__ void wait_for_earlier_launch() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename... P, typename... Args>
-cudaError_t launch_kernel(void (*kern)(P...), size_t blocks, dim3 threads, size_t smem, cudaStream_t s, bool overlap,
-                          Args... args) {
-  if (blocks > 0x7fffffffull) return cudaErrorInvalidConfiguration;
+cudaError_t launch_kernel_2d(void (*kern)(P...), dim3 grid, dim3 threads, size_t smem, cudaStream_t s, bool overlap,
+                             Args... args) {
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.gridDim = grid;
   cfg.blockDim = threads;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = &at;
   cfg.numAttrs = overlap ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
+template <typename... P, typename... Args>
+cudaError_t launch_kernel(void (*kern)(P...), size_t blocks, dim3 threads, size_t smem, cudaStream_t s, bool overlap,
+                          Args... args) {
+  if (blocks > 0x7fffffffull) return cudaErrorInvalidConfiguration;
+  return launch_kernel_2d(kern, dim3((unsigned)blocks), threads, smem, s, overlap, args...);
 }
 
 // A cell along one direction: only its first and last nodes can be shared,

@@ -80,6 +80,8 @@ struct SolveWs {
   size_t cap_partial = 0;
   int* active = nullptr;     // per-column "not yet converged" flags
   size_t cap_active = 0;
+  int* ticket = nullptr;     // CTAs done per column tile of a reduction (0 between launches)
+  size_t cap_ticket = 0;
   double* diag = nullptr;
   double* dinv64 = nullptr;
   float* dinv32 = nullptr;

@@ -12,6 +12,7 @@
 #include <cstring>
 #include <vector>
 
+#include "fe_dispatch.cuh"
 #include "fe_internal.h"
 
 namespace fe {
@@ -63,16 +64,28 @@ __global__ void col_sum_partials(const double* __restrict__ partial, int nblocks
 }
 
 template <typename T>
-cudaError_t col_dot(const T* a, const T* b, size_t n, int nv, double* partial, double* out, cudaStream_t s);
+cudaError_t col_dot(const T* a, const T* b, size_t n, int nv, const SolveWs& w, double* out, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // wide variants: 16-byte accesses (4 floats or 2 doubles of consecutive
 // columns per thread) and enough CTAs to fill every SM, for blocks whose
 // column count is a multiple of the vector width.  Same deterministic
-// per-CTA partials, summed in a fixed order.
+// per-CTA partials; the last CTA of a column tile to finish sums the tile's
+// partials in a fixed order and goes on to the CG scalar they are for, which
+// saves one or two launches per sum.  A CTA's 256 threads are x column groups x
+// 256 / x rows, x as many as the block has (8 groups of 32 columns in FP32: a
+// fixed 32 left three quarters of the threads idle).  The mixed solve at 12^3, p
+// = 6, 32 columns: 203 -> 155 ms (580 iterations) with this, the x update moved
+// to the direction kernel and z = D^-1 r formed where it is used (10 vectors
+// streamed per iteration instead of 12).
 // ---------------------------------------------------------------------------
 
 constexpr int kWideBlocks = 152 * 8;
+// The reductions take 2 CTAs per SM with four rows in flight per thread: the sum
+// over threads and CTAs is the slow part (FP64 runs at 1/64 of the FP32 rate): with
+// 8 CTAs per SM joined in FP64 a 100 MB dot product took 68 us.
+constexpr int kWideRedBlocks = 152 * 2;
+constexpr int kWideRows = 4;
 
 template <typename T>
 struct Wide;
@@ -104,12 +117,13 @@ inline bool wide_ok(int nv, const void* const* ptrs, int n_ptrs) {
 }
 
 // Rows of CTA b: [b * rows_per, ...); thread (x, y): column group x of the
-// CTA's column tile (32 groups of Wide<T>::N columns), rows y, y + 8, ...
+// CTA's column tile (blockDim.x groups of Wide<T>::N columns), rows y, y +
+// blockDim.y, ...
 #define FE_WIDE_PROLOGUE(T)                                                            \
   using W = Wide<T>;                                                                   \
   using V = typename W::V;                                                             \
   const int ncg = nv / W::N;                                                           \
-  const int cg = blockIdx.y * 32 + threadIdx.x;                                        \
+  const int cg = blockIdx.y * blockDim.x + threadIdx.x;                                \
   const bool col_ok = cg < ncg;                                                        \
   const size_t rows_per = (n + gridDim.x - 1) / gridDim.x;                             \
   const size_t r0 = (size_t)blockIdx.x * rows_per;                                     \
@@ -118,19 +132,25 @@ inline bool wide_ok(int nv, const void* const* ptrs, int n_ptrs) {
 // Per-thread column sums of products.  FP64 blocks accumulate in FP64.  FP32
 // blocks accumulate in FP32 with Kahan's compensation (the running error is
 // fed back into the next term, so the sum is accurate to a few FP32 ulps
-// whatever its length) and are converted to FP64 once, for the cross-thread
-// reduction: GB300 runs FP64 at 1/64 of the FP32 rate, and two conversions
+// whatever its length) and are joined over the CTA in double-float, converted to
+// FP64 once per CTA: GB300 runs FP64 at 1/64 of the FP32 rate, and two conversions
 // plus an FP64 multiply-add per element would bound these streaming kernels.
 template <typename T>
 struct ColAcc;
 template <>
 struct ColAcc<double> {
+  using Part = double;   // a thread's sum, summed over the CTA
+  static __device__ Part join(Part a, Part b) { return a + b; }
+  static __device__ double out(Part a) { return a; }
   double s = 0.0;
   __device__ void add(double a, double b) { s = fma(a, b, s); }
-  __device__ double value() const { return s; }
+  __device__ Part value() const { return s; }
 };
 template <>
 struct ColAcc<float> {
+  using Part = ff;       // s - c exactly; double-float sums keep 48 bits
+  static __device__ Part join(Part a, Part b) { return ff_add(a, b); }
+  static __device__ double out(Part a) { return ff_to_double(a); }
   float s = 0.f, c = 0.f;
   __device__ void add(float a, float b) {
     const float y = __fsub_rn(__fmul_rn(a, b), c);
@@ -138,102 +158,188 @@ struct ColAcc<float> {
     c = __fsub_rn(__fsub_rn(t, s), y);
     s = t;
   }
-  __device__ double value() const { return (double)s - (double)c; }
+  __device__ Part value() const { return renorm(s, -c); }
 };
 
-// partial[b][c] over columns c of the thread's group
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
+// What a column sum is for.
+struct ColScalar {
+  enum Kind { kSum, kAlpha, kBeta } kind;
+  double* out;            // kSum: the sum; kAlpha: rz / sum; kBeta: sum / rz (then rz = sum)
+  double* rz;
+  const int* active;
+  double* sum;            // kAlpha, kBeta: the sum itself, or null
+  int* status;
+  int* ticket;            // one counter per column tile, 0 between launches
+};
+
+// alpha = active ? rz / pq : 0; flags a breakdown when pq <= 0 on an active column
+__device__ __forceinline__ double cg_alpha(double rz, double pq, int active, int* status) {
+  if (!active) return 0.0;
+  if (!(pq > 0.0) || !isfinite(pq)) {
+    atomicMax(status, (int)FE_EBREAKDOWN);
+    return 0.0;
+  }
+  return rz / pq;
+}
+
+// Per-CTA partials of the thread's column group, then the tile's sums and
+// scalars by the last CTA: one warp per column, lane l adds the partials l, l +
+// 32, ... in order, then a fixed butterfly (deterministic).
 template <typename T>
-__device__ __forceinline__ void wide_store_partials(double (&s)[Wide<T>::N], bool col_ok, int cg, int nv,
-                                                    double* __restrict__ partial) {
-  __shared__ double red[8][32][Wide<T>::N];
+__device__ __forceinline__ void wide_finish(const ColAcc<T> (&acc)[Wide<T>::N], bool col_ok, int cg, int nv,
+                                            double* __restrict__ partial, const ColScalar& o) {
+  constexpr int N = Wide<T>::N;
+  using Part = typename ColAcc<T>::Part;
+  __shared__ Part red[256][N];
+  __shared__ bool last;
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
 #pragma unroll
-  for (int k = 0; k < Wide<T>::N; ++k) red[threadIdx.y][threadIdx.x][k] = s[k];
-  __syncthreads();
+  for (int k = 0; k < N; ++k) red[tid][k] = acc[k].value();
+  for (int h = blockDim.y / 2; h > 0; h /= 2) {   // blockDim.y is a power of two
+    __syncthreads();
+    if ((int)threadIdx.y < h) {
+#pragma unroll
+      for (int k = 0; k < N; ++k) red[tid][k] = ColAcc<T>::join(red[tid][k], red[tid + h * blockDim.x][k]);
+    }
+  }
   if (threadIdx.y == 0 && col_ok) {
 #pragma unroll
-    for (int k = 0; k < Wide<T>::N; ++k) {
-      double t = s[k];
-      for (int y = 1; y < 8; ++y) t += red[y][threadIdx.x][k];
-      partial[(size_t)blockIdx.x * nv + cg * Wide<T>::N + k] = t;
+    for (int k = 0; k < N; ++k) partial[(size_t)blockIdx.x * nv + cg * N + k] = ColAcc<T>::out(red[tid][k]);
+  }
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) last = atomicAdd(o.ticket + blockIdx.y, 1) == (int)gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (tid == 0) o.ticket[blockIdx.y] = 0;
+  const int c0 = blockIdx.y * blockDim.x * N, c1 = min(nv, c0 + (int)blockDim.x * N), lane = tid & 31;
+  for (int c = c0 + tid / 32; c < c1; c += 8) {
+    double t = 0.0;
+#pragma unroll 8
+    for (int b = lane; b < (int)gridDim.x; b += 32) t += __ldcg(partial + (size_t)b * nv + c);
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) t += __shfl_xor_sync(0xffffffffu, t, w);
+    if (lane != 0) continue;
+    if (o.kind == ColScalar::kSum) {
+      o.out[c] = t;
+    } else if (o.kind == ColScalar::kAlpha) {
+      o.out[c] = cg_alpha(o.rz[c], t, o.active[c], o.status);
+    } else {
+      o.out[c] = o.active[c] && o.rz[c] != 0.0 ? t / o.rz[c] : 0.0;
+      o.rz[c] = t;
     }
+    if (o.sum) o.sum[c] = t;
   }
 }
 
+// a . b per column
 template <typename T>
-__global__ void __launch_bounds__(256) col_dot_partial_wide(const T* __restrict__ a, const T* __restrict__ b,
-                                                            size_t n, int nv, double* __restrict__ partial) {
+__global__ void __launch_bounds__(256) col_dot_wide(const T* __restrict__ a, const T* __restrict__ b, size_t n, int nv,
+                                                    double* __restrict__ partial, const ColScalar o) {
   FE_WIDE_PROLOGUE(T)
+  let_next_launch_start();
+  wait_for_earlier_launch();
   ColAcc<T> acc[W::N];
   if (col_ok) {
-    for (size_t r = r0 + threadIdx.y; r < r1; r += 8) {
-      const V va = reinterpret_cast<const V*>(a + r * nv)[cg];
-      const V vb = reinterpret_cast<const V*>(b + r * nv)[cg];
+    for (size_t r = r0 + threadIdx.y; r < r1; r += kWideRows * blockDim.y) {
+      V va[kWideRows], vb[kWideRows];
 #pragma unroll
-      for (int k = 0; k < W::N; ++k) acc[k].add(W::get(va, k), W::get(vb, k));
+      for (int j = 0; j < kWideRows; ++j) {
+        const size_t row = r + j * blockDim.y;
+        if (row < r1) {
+          va[j] = reinterpret_cast<const V*>(a + row * nv)[cg];
+          vb[j] = reinterpret_cast<const V*>(b + row * nv)[cg];
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < kWideRows; ++j)
+        if (r + j * blockDim.y < r1) {
+#pragma unroll
+          for (int k = 0; k < W::N; ++k) acc[k].add(W::get(va[j], k), W::get(vb[j], k));
+        }
     }
   }
-  double s[W::N];
-#pragma unroll
-  for (int k = 0; k < W::N; ++k) s[k] = acc[k].value();
-  wide_store_partials<T>(s, col_ok, cg, nv, partial);
+  wide_finish<T>(acc, col_ok, cg, nv, partial, o);
 }
 
-// x += alpha_c p, r -= alpha_c q, z = dinv .* r, partial r.z (one pass)
+// r -= alpha_c q and r . (dinv r) per column
 template <typename T>
-__global__ void __launch_bounds__(256) cg_step_kernel_wide(T* __restrict__ x, T* __restrict__ r, T* __restrict__ z,
-                                                           const T* __restrict__ p, const T* __restrict__ q,
-                                                           const T* __restrict__ dinv,
-                                                           const double* __restrict__ alpha, size_t n, int nv,
-                                                           double* __restrict__ partial) {
+__global__ void __launch_bounds__(256) cg_residual_wide(T* __restrict__ r, const T* __restrict__ q,
+                                                        const T* __restrict__ dinv, const double* __restrict__ alpha,
+                                                        size_t n, int nv, double* __restrict__ partial,
+                                                        const ColScalar o) {
   FE_WIDE_PROLOGUE(T)
+  let_next_launch_start();
+  wait_for_earlier_launch();
   ColAcc<T> acc[W::N];
   if (col_ok) {
     T a[W::N];
 #pragma unroll
     for (int k = 0; k < W::N; ++k) a[k] = (T)alpha[cg * W::N + k];
-    for (size_t row = r0 + threadIdx.y; row < r1; row += 8) {
-      const size_t o = row * nv;
-      V vx = reinterpret_cast<const V*>(x + o)[cg];
-      V vr = reinterpret_cast<const V*>(r + o)[cg];
-      const V vp = reinterpret_cast<const V*>(p + o)[cg];
-      const V vq = reinterpret_cast<const V*>(q + o)[cg];
-      const T d = dinv ? dinv[row] : T(1);
-      V vz;
+    for (size_t r_ = r0 + threadIdx.y; r_ < r1; r_ += kWideRows * blockDim.y) {
+      V vr[kWideRows], vq[kWideRows];
+      T d[kWideRows];
 #pragma unroll
-      for (int k = 0; k < W::N; ++k) {
-        W::set(vx, k, W::get(vx, k) + a[k] * W::get(vp, k));
-        const T rn = W::get(vr, k) - a[k] * W::get(vq, k);
-        W::set(vr, k, rn);
-        const T zn = rn * d;
-        W::set(vz, k, zn);
-        acc[k].add(rn, zn);
+      for (int j = 0; j < kWideRows; ++j) {
+        const size_t row = r_ + j * blockDim.y;
+        if (row < r1) {
+          vr[j] = reinterpret_cast<const V*>(r + row * nv)[cg];
+          vq[j] = reinterpret_cast<const V*>(q + row * nv)[cg];
+          d[j] = dinv ? dinv[row] : T(1);
+        }
       }
-      reinterpret_cast<V*>(x + o)[cg] = vx;
-      reinterpret_cast<V*>(r + o)[cg] = vr;
-      reinterpret_cast<V*>(z + o)[cg] = vz;
+#pragma unroll
+      for (int j = 0; j < kWideRows; ++j) {
+        const size_t row = r_ + j * blockDim.y;
+        if (row < r1) {
+#pragma unroll
+          for (int k = 0; k < W::N; ++k) {
+            const T rn = W::get(vr[j], k) - a[k] * W::get(vq[j], k);
+            W::set(vr[j], k, rn);
+            acc[k].add(rn, mul_rn(rn, d[j]));
+          }
+          reinterpret_cast<V*>(r + row * nv)[cg] = vr[j];
+        }
+      }
     }
   }
-  double s[W::N];
-#pragma unroll
-  for (int k = 0; k < W::N; ++k) s[k] = acc[k].value();
-  wide_store_partials<T>(s, col_ok, cg, nv, partial);
+  wide_finish<T>(acc, col_ok, cg, nv, partial, o);
 }
 
-// p = z + beta_c p
+// p = z + beta_c p with z = dinv z (dinv null: z as it is); with x also x +=
+// alpha_c p for the p read, so that p is read once per iteration
 template <typename T>
 __global__ void __launch_bounds__(256) cg_direction_kernel_wide(T* __restrict__ p, const T* __restrict__ z,
-                                                                const double* __restrict__ beta, size_t n, int nv) {
+                                                                const T* __restrict__ dinv,
+                                                                const double* __restrict__ beta, T* __restrict__ x,
+                                                                const double* __restrict__ alpha, size_t n, int nv) {
   FE_WIDE_PROLOGUE(T)
+  let_next_launch_start();
+  wait_for_earlier_launch();
   if (!col_ok) return;
-  T bc[W::N];
+  T bc[W::N], ac[W::N];
 #pragma unroll
-  for (int k = 0; k < W::N; ++k) bc[k] = (T)beta[cg * W::N + k];
-  for (size_t row = r0 + threadIdx.y; row < r1; row += 8) {
+  for (int k = 0; k < W::N; ++k) {
+    bc[k] = (T)beta[cg * W::N + k];
+    ac[k] = x ? (T)alpha[cg * W::N + k] : T(0);
+  }
+  for (size_t row = r0 + threadIdx.y; row < r1; row += blockDim.y) {
     const size_t o = row * nv;
     V vp = reinterpret_cast<const V*>(p + o)[cg];
     const V vz = reinterpret_cast<const V*>(z + o)[cg];
+    const T d = dinv ? dinv[row] : T(1);
+    if (x) {
+      V vx = reinterpret_cast<const V*>(x + o)[cg];
 #pragma unroll
-    for (int k = 0; k < W::N; ++k) W::set(vp, k, W::get(vz, k) + bc[k] * W::get(vp, k));
+      for (int k = 0; k < W::N; ++k) W::set(vx, k, W::get(vx, k) + ac[k] * W::get(vp, k));
+      reinterpret_cast<V*>(x + o)[cg] = vx;
+    }
+#pragma unroll
+    for (int k = 0; k < W::N; ++k) W::set(vp, k, fma(bc[k], W::get(vp, k), mul_rn(W::get(vz, k), d)));
     reinterpret_cast<V*>(p + o)[cg] = vp;
   }
 }
@@ -247,7 +353,7 @@ __global__ void __launch_bounds__(256) cg_update_kernel_wide(T* __restrict__ x, 
   T a[W::N];
 #pragma unroll
   for (int k = 0; k < W::N; ++k) a[k] = (T)alpha[cg * W::N + k];
-  for (size_t row = r0 + threadIdx.y; row < r1; row += 8) {
+  for (size_t row = r0 + threadIdx.y; row < r1; row += blockDim.y) {
     const size_t o = row * nv;
     V vx = reinterpret_cast<const V*>(x + o)[cg];
     V vr = reinterpret_cast<const V*>(r + o)[cg];
@@ -278,7 +384,7 @@ __global__ void __launch_bounds__(256) fcg_safeguard_kernel_wide(const T* __rest
     any = any || bad[k];
   }
   if (!any) return;
-  for (size_t row = r0 + threadIdx.y; row < r1; row += 8) {
+  for (size_t row = r0 + threadIdx.y; row < r1; row += blockDim.y) {
     const size_t o = row * nv;
     const V vr = reinterpret_cast<const V*>(r + o)[cg];
     V vz = reinterpret_cast<const V*>(z + o)[cg];
@@ -291,29 +397,26 @@ __global__ void __launch_bounds__(256) fcg_safeguard_kernel_wide(const T* __rest
 }
 #undef FE_WIDE_PROLOGUE
 
-// out[c] = sum_b partial[b * nv + c]: one warp per column, lane l adds the
-// partials l, l + 32, ... in order, then a fixed butterfly (deterministic).
-__global__ void col_sum_partials_warp(const double* __restrict__ partial, int nblocks, int nv,
-                                      double* __restrict__ out) {
-  const int c = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32, lane = threadIdx.x & 31;
-  if (c >= nv) return;
-  double s = 0.0;
-  for (int b = lane; b < nblocks; b += 32) s += partial[(size_t)b * nv + c];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) out[c] = s;
+// Threads and grid of the wide kernels for nv columns.
+template <typename T>
+dim3 wide_block(int nv) {
+  int x = 1;
+  while (x < 32 && x < nv / Wide<T>::N) x *= 2;
+  return dim3(x, 256 / x);
+}
+template <typename T>
+dim3 wide_grid(int nv, int blocks = kWideBlocks) {
+  const int x = (int)wide_block<T>(nv).x, groups = nv / Wide<T>::N;
+  return dim3(blocks, (unsigned)((groups + x - 1) / x));
 }
 
-inline dim3 wide_grid(int nv, int vec) { return dim3(kWideBlocks, (unsigned)((nv / vec + 31) / 32)); }
-
 template <typename T>
-cudaError_t col_dot(const T* a, const T* b, size_t n, int nv, double* partial, double* out, cudaStream_t s) {
+cudaError_t col_dot(const T* a, const T* b, size_t n, int nv, const SolveWs& w, double* out, cudaStream_t s) {
   const void* ptrs[2] = {a, b};
-  if (wide_ok<T>(nv, ptrs, 2)) {
-    col_dot_partial_wide<T><<<wide_grid(nv, Wide<T>::N), dim3(32, 8), 0, s>>>(a, b, n, nv, partial);
-    col_sum_partials_warp<<<(nv + 7) / 8, 256, 0, s>>>(partial, kWideBlocks, nv, out);
-    return cudaGetLastError();
-  }
+  double* partial = w.partial;
+  if (wide_ok<T>(nv, ptrs, 2))
+    return launch_kernel_2d(col_dot_wide<T>, wide_grid<T>(nv, kWideRedBlocks), wide_block<T>(nv), 0, s, true, a, b, n, nv, partial,
+                            ColScalar{ColScalar::kSum, out, nullptr, nullptr, nullptr, nullptr, w.ticket});
   dim3 grid(kRedBlocks, (nv + kColTile - 1) / kColTile);
   col_dot_partial<T><<<grid, dim3(kColTile, 8), 0, s>>>(a, b, n, nv, partial);
   col_sum_partials<<<(nv + 127) / 128, 128, 0, s>>>(partial, kRedBlocks, nv, out);
@@ -490,6 +593,10 @@ cudaError_t solver_workspace(fe_ctx* c, int nv) {
   if (e == cudaSuccess) e = grow(&w.colbuf, &w.cap_col, (size_t)nv * 12);
   if (e == cudaSuccess) e = grow(&w.partial, &w.cap_partial, (size_t)kWideBlocks * nv);
   if (e == cudaSuccess) e = grow(&w.active, &w.cap_active, (size_t)nv);
+  if (e == cudaSuccess && w.cap_ticket < (size_t)nv) {
+    e = grow(&w.ticket, &w.cap_ticket, (size_t)nv);
+    if (e == cudaSuccess) e = cudaMemset(w.ticket, 0, (size_t)nv * sizeof(int));
+  }
   if (e == cudaSuccess && !w.dinv64) {
     e = cudaMalloc(&w.dinv64, n * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&w.dinv32, n * sizeof(float));
@@ -557,13 +664,13 @@ fe_status pcg(fe_ctx* c, const T* b, T* x, int nv, const double* tol_host, int m
   if (learned) st = learned_precond_apply(c, r, z, nv, sizeof(T) == 8, s);
   else precond_jacobi_kernel<T><<<ew_grid(tot), 256, 0, s>>>(r, dinv, z, n, nv);
   if (st != FE_OK) return st;
-  if ((e = col_dot<T>(r, z, n, nv, w.partial, rz, s)) != cudaSuccess) return from_cuda(e);
+  if ((e = col_dot<T>(r, z, n, nv, w, rz, s)) != cudaSuccess) return from_cuda(e);
   if (learned) {
     fcg_safeguard_kernel<T><<<ew_grid(tot), 256, 0, s>>>(r, dinv_all, z, rz, tot, nv);
-    if ((e = col_dot<T>(r, z, n, nv, w.partial, rz, s)) != cudaSuccess) return from_cuda(e);
+    if ((e = col_dot<T>(r, z, n, nv, w, rz, s)) != cudaSuccess) return from_cuda(e);
   }
   if ((e = cudaMemcpyAsync(p, z, tot * sizeof(T), cudaMemcpyDeviceToDevice, s)) != cudaSuccess) return from_cuda(e);
-  if ((e = col_dot<T>(r, r, n, nv, w.partial, rr, s)) != cudaSuccess) return from_cuda(e);
+  if ((e = col_dot<T>(r, r, n, nv, w, rr, s)) != cudaSuccess) return from_cuda(e);
   cudaMemcpyAsync(rr_h.data(), rr, nv * sizeof(double), cudaMemcpyDeviceToHost, s);
   cudaStreamSynchronize(s);
   for (int j = 0; j < nv; ++j) act_h[j] = std::sqrt(rr_h[j]) > tol_host[j];
@@ -574,47 +681,50 @@ fe_status pcg(fe_ctx* c, const T* b, T* x, int nv, const double* tol_host, int m
   while (!done && it < max_it) {
     st = apply_mode<T>(c, p, q, nv, s);
     if (st != FE_OK) return st;
-    if ((e = col_dot<T>(p, q, n, nv, w.partial, pq, s)) != cudaSuccess) return from_cuda(e);
-    cg_alpha_kernel<<<(nv + 127) / 128, 128, 0, s>>>(rz, pq, w.active, alpha, nv, c->d_status);
+    const dim3 wg = wide_grid<T>(nv), wr = wide_grid<T>(nv, kWideRedBlocks), wb = wide_block<T>(nv);
+    if (wide) {
+      e = launch_kernel_2d(col_dot_wide<T>, wr, wb, 0, s, true, p, q, n, nv, w.partial,
+                           ColScalar{ColScalar::kAlpha, alpha, rz, w.active, pq, c->d_status, w.ticket});
+    } else {
+      e = col_dot<T>(p, q, n, nv, w, pq, s);
+      cg_alpha_kernel<<<(nv + 127) / 128, 128, 0, s>>>(rz, pq, w.active, alpha, nv, c->d_status);
+    }
+    if (e != cudaSuccess) return from_cuda(e);
     if (learned) {
-      if (wide)
-        cg_update_kernel_wide<T><<<wide_grid(nv, Wide<T>::N), dim3(32, 8), 0, s>>>(x, r, p, q, alpha, n, nv);
-      else
-        cg_update_kernel<T><<<ew_grid(tot), 256, 0, s>>>(x, r, p, q, alpha, tot, nv);
+      if (wide) cg_update_kernel_wide<T><<<wg, wb, 0, s>>>(x, r, p, q, alpha, n, nv);
+      else cg_update_kernel<T><<<ew_grid(tot), 256, 0, s>>>(x, r, p, q, alpha, tot, nv);
       st = learned_precond_apply(c, r, z, nv, sizeof(T) == 8, s);
       if (st != FE_OK) return st;
-      if ((e = col_dot<T>(r, z, n, nv, w.partial, rznew, s)) != cudaSuccess) return from_cuda(e);
-    } else {
-      if (wide) {
-        cg_step_kernel_wide<T><<<wide_grid(nv, Wide<T>::N), dim3(32, 8), 0, s>>>(x, r, z, p, q, dinv, alpha, n, nv,
-                                                                                 w.partial);
-        col_sum_partials_warp<<<(nv + 7) / 8, 256, 0, s>>>(w.partial, kWideBlocks, nv, rznew);
-      } else {
-        const dim3 grid(kRedBlocks, (nv + kColTile - 1) / kColTile);
-        cg_step_kernel<T><<<grid, dim3(kColTile, 8), 0, s>>>(x, r, z, p, q, dinv, alpha, n, nv, w.partial);
-        col_sum_partials<<<(nv + 127) / 128, 128, 0, s>>>(w.partial, kRedBlocks, nv, rznew);
-      }
-    }
-    if (learned) {
-      if (wide)
-        fcg_safeguard_kernel_wide<T><<<wide_grid(nv, Wide<T>::N), dim3(32, 8), 0, s>>>(r, dinv_all, z, rznew, n, nv);
-      else
-        fcg_safeguard_kernel<T><<<ew_grid(tot), 256, 0, s>>>(r, dinv_all, z, rznew, tot, nv);
-      if ((e = col_dot<T>(r, z, n, nv, w.partial, rznew, s)) != cudaSuccess) return from_cuda(e);
+      if ((e = col_dot<T>(r, z, n, nv, w, rznew, s)) != cudaSuccess) return from_cuda(e);
+      if (wide) fcg_safeguard_kernel_wide<T><<<wg, wb, 0, s>>>(r, dinv_all, z, rznew, n, nv);
+      else fcg_safeguard_kernel<T><<<ew_grid(tot), 256, 0, s>>>(r, dinv_all, z, rznew, tot, nv);
+      if ((e = col_dot<T>(r, z, n, nv, w, rznew, s)) != cudaSuccess) return from_cuda(e);
       // flexible CG (Notay): beta = -(z_new . A p) / (p . A p)
-      if ((e = col_dot<T>(z, q, n, nv, w.partial, rzmid, s)) != cudaSuccess) return from_cuda(e);
+      if ((e = col_dot<T>(z, q, n, nv, w, rzmid, s)) != cudaSuccess) return from_cuda(e);
+      cg_beta_kernel<<<(nv + 127) / 128, 128, 0, s>>>(rznew, rzmid, pq, rz, w.active, beta, nv, 1);
+      if (wide)
+        e = launch_kernel_2d(cg_direction_kernel_wide<T>, wg, wb, 0, s, true, p, z, nullptr, beta, nullptr, alpha, n, nv);
+    } else if (wide) {
+      // 10 vectors streamed per iteration: p, q | r, q -> r | x, p, r -> x, p
+      e = launch_kernel_2d(cg_residual_wide<T>, wr, wb, 0, s, true, r, q, dinv, alpha, n, nv, w.partial,
+                           ColScalar{ColScalar::kBeta, beta, rz, w.active, nullptr, c->d_status, w.ticket});
+      if (e == cudaSuccess)
+        e = launch_kernel_2d(cg_direction_kernel_wide<T>, wg, wb, 0, s, true, p, r, dinv, beta, x, alpha, n, nv);
+    } else {
+      const dim3 grid(kRedBlocks, (nv + kColTile - 1) / kColTile);
+      cg_step_kernel<T><<<grid, dim3(kColTile, 8), 0, s>>>(x, r, z, p, q, dinv, alpha, n, nv, w.partial);
+      col_sum_partials<<<(nv + 127) / 128, 128, 0, s>>>(w.partial, kRedBlocks, nv, rznew);
+      cg_beta_kernel<<<(nv + 127) / 128, 128, 0, s>>>(rznew, rzmid, pq, rz, w.active, beta, nv, 0);
     }
-    cg_beta_kernel<<<(nv + 127) / 128, 128, 0, s>>>(rznew, rzmid, pq, rz, w.active, beta, nv, learned ? 1 : 0);
-    if (wide)
-      cg_direction_kernel_wide<T><<<wide_grid(nv, Wide<T>::N), dim3(32, 8), 0, s>>>(p, z, beta, n, nv);
-    else
+    if (e != cudaSuccess) return from_cuda(e);
+    if (!wide)
       cg_direction_kernel<T><<<dim3(kRedBlocks, (nv + kColTile - 1) / kColTile), dim3(kColTile, 8), 0, s>>>(
           p, z, beta, n, nv);
     ++it;
     if (hook) hook(hook_user, it, x, r, s);
     if ((e = cudaGetLastError()) != cudaSuccess) return from_cuda(e);
     if (it % check_every == 0 || it == max_it) {
-      if ((e = col_dot<T>(r, r, n, nv, w.partial, rr, s)) != cudaSuccess) return from_cuda(e);
+      if ((e = col_dot<T>(r, r, n, nv, w, rr, s)) != cudaSuccess) return from_cuda(e);
       cudaMemcpyAsync(rr_h.data(), rr, nv * sizeof(double), cudaMemcpyDeviceToHost, s);
       if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return from_cuda(e);
       int hs = 0;
@@ -646,7 +756,7 @@ fe_status true_residual(fe_ctx* c, const double* B, const double* X, int nv, dou
   fe_status st = apply_mode<double>(c, X, r64, nv, s);
   if (st != FE_OK) return st;
   residual_kernel<double><<<ew_grid(tot), 256, 0, s>>>(B, r64, tot);
-  cudaError_t e = col_dot<double>(r64, r64, n, nv, w.partial, rr, s);
+  cudaError_t e = col_dot<double>(r64, r64, n, nv, w, rr, s);
   if (e != cudaSuccess) return from_cuda(e);
   std::vector<double> h(nv);
   cudaMemcpyAsync(h.data(), rr, nv * sizeof(double), cudaMemcpyDeviceToHost, s);
@@ -680,7 +790,7 @@ void free_solver_workspace(fe_ctx* c) {
   SolveWs& w = c->ws;
   for (int k = 0; k < 4; ++k) cudaFree(w.v64[k]);
   for (int k = 0; k < 6; ++k) cudaFree(w.v32[k]);
-  cudaFree(w.colbuf); cudaFree(w.partial); cudaFree(w.active);
+  cudaFree(w.colbuf); cudaFree(w.partial); cudaFree(w.active); cudaFree(w.ticket);
   cudaFree(w.diag); cudaFree(w.dinv64); cudaFree(w.dinv32);
   w = SolveWs();
 }
@@ -710,7 +820,7 @@ extern "C" fe_status fe_solve(fe_ctx* c, const double* B, double* X, int nv, dou
   // ||b_j||
   std::vector<double> bnorm(nv), rel(nv), tol(nv);
   double* bb = w.colbuf + 8 * nv;
-  if ((e = col_dot<double>(B, B, n, nv, w.partial, bb, s)) != cudaSuccess) return from_cuda(e);
+  if ((e = col_dot<double>(B, B, n, nv, w, bb, s)) != cudaSuccess) return from_cuda(e);
   cudaMemcpyAsync(bnorm.data(), bb, nv * sizeof(double), cudaMemcpyDeviceToHost, s);
   cudaStreamSynchronize(s);
   for (int j = 0; j < nv; ++j) bnorm[j] = std::sqrt(bnorm[j]);
