@@ -98,10 +98,12 @@ struct MlpArgs {
 //               BF16 pairs to tensor memory, sum of squares; GEMM1
 //   warps 8-15  hidden layer (1/s, b1, ReLU), GEMM2 in chunks of 128 outputs
 //               alternating between the accumulators, scatter
-// What bounds it: the issue of the gather's and scatter's 128-byte loads (a
-// warp's 32 independent loads take 4-7 K cycles to issue, the wait for their
-// data 1 K more); the tensor pipe is idle.  One application on 24^3 cells, p =
-// 6, 128 columns: 6.37 -> 3.18 ms (24^3, p = 4, 100 columns 2.28 -> 1.25 ms)
+// What bounds it: the issue of the gather's and scatter's loads (with one column
+// per lane, a warp's 32 independent 128-byte loads take 4-7 K cycles to issue and
+// their data 1 K more to arrive), so where rows allow (WIDE) a lane moves 16 bytes,
+// four nodes x 32 columns per access, and a warp transposes through 1 KB of
+// shared memory; the tensor pipe is idle.  One application on 24^3 cells, p = 6,
+// 128 columns: 6.4 -> 2.05 ms (127 columns, one column per lane: 6.4 -> 3.13 ms)
 // against a kernel that reloaded both images into one 218 KB CTA per task, with
 // gather, GEMMs and scatter taking turns and z initialised in a pass of its own.
 constexpr int kMlpThreads = 512;
@@ -142,19 +144,24 @@ struct alignas(16) MlpNode {
   float w, d;       // partition-of-unity weight; 1 / D for a first colour, else 1
 };
 
+constexpr int kStageRow = 36;   // 32 columns of a node, 16-byte rows in different banks
+
 struct MlpShared {
   unsigned char *w1, *w2;
   MlpNode* node;     // [2][K1]
   float* b2;         // [K1]
+  float* stage;      // [16 warps][8 nodes][kStageRow]: a warp's transposes (WIDE)
   float* ssq;        // [2][2][128]: partial squared norms
   uint64_t* bar;     // GEMM1 done, GEMM2 chunks 0..2 done, task's accumulators read
   uint32_t* tslot;
 };
 
 __host__ __device__ constexpr size_t mlp_smem_bytes(int K1) {
-  return (size_t)2 * kTile * K1 * 2 + (size_t)K1 * (2 * sizeof(MlpNode) + 4) + 4 * kTile * sizeof(float) + 6 * 8 + 16;
+  return (size_t)2 * kTile * K1 * 2 + (size_t)K1 * (2 * sizeof(MlpNode) + 4) + 4 * kTile * sizeof(float) + 6 * 8 + 16 +
+         (size_t)kMlpThreads / 32 * 8 * kStageRow * sizeof(float);
 }
 
+template <bool WIDE>
 __global__ void __launch_bounds__(kMlpThreads, 1) mlp_precond_kernel(const MlpArgs a, const MeshDev m,
                                                                      const int* __restrict__ cells, int n_tasks,
                                                                      const float* __restrict__ R,
@@ -166,7 +173,8 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_precond_kernel(const MlpAr
   MlpShared sh;
   sh.w1 = smem;
   sh.w2 = smem + img;
-  sh.node = reinterpret_cast<MlpNode*>(smem + 2 * img);
+  sh.stage = reinterpret_cast<float*>(smem + 2 * img);
+  sh.node = reinterpret_cast<MlpNode*>(sh.stage + kMlpThreads / 32 * 8 * kStageRow);
   sh.b2 = reinterpret_cast<float*>(sh.node + 2 * K1);
   sh.bar = reinterpret_cast<uint64_t*>(sh.b2 + K1);
   sh.ssq = reinterpret_cast<float*>(sh.bar + 6);
@@ -175,6 +183,8 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_precond_kernel(const MlpAr
 
   const int t = threadIdx.x, warp = t >> 5;
   const int row = t & (kTile - 1), half = (t >> 7) & 1;
+  // WIDE: a warp moves four nodes x 32 columns per access, lane = (node wj, columns wc ... + 3)
+  const int wj = (t & 31) >> 3, wc = (t & 7) * 4;
   const int n_chunks = (K1 + 127) / 128;
   const int P = a.np - 1;
 
@@ -200,6 +210,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_precond_kernel(const MlpAr
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *sh.tslot;
+  float* stage = sh.stage + warp * 8 * kStageRow;
   const uint32_t lane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
   bool ok = true;
 
@@ -245,27 +256,52 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_precond_kernel(const MlpAr
       ok = barrier_and(1, kMlpHalf, ok);
       if (!ok) break;
       const int col = (task % n_cb) * kTile + row;
+      const int col4 = (task % n_cb) * kTile + (warp & 3) * 32 + wc;
       const bool active = col < n_vec;
       const MlpNode* node = sh.node + buf * K1;
       float ss = 0.f;
       // 8-node chunks kg = half, half + 2, ...; four chunks' loads at once
       for (int k0 = half; k0 < K1 / 8; k0 += 8) {
         float v[4][8];
+        if constexpr (WIDE) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+          for (int j = 0; j < 4; ++j)
 #pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int i = (k0 + 2 * j) * 8 + u;
-            v[j][u] = 0.f;
-            const long long nd = i < K1 ? node[i].code : -1;
-            if (active && nd >= 0 && !(nd & 1)) v[j][u] = __ldg(R + (nd >> 2) * n_vec + col);
-          }
+            for (int q = 0; q < 2; ++q) {   // nodes wj and wj + 4 of chunk k0 + 2 j
+              const int i = (k0 + 2 * j) * 8 + 4 * q + wj;
+              const long long nd = i < K1 ? node[i].code : -1;
+              float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+              if (col4 < n_vec && nd >= 0 && !(nd & 1))
+                x = __ldg(reinterpret_cast<const float4*>(R + (nd >> 2) * n_vec + col4));
+              v[j][4 * q] = x.x; v[j][4 * q + 1] = x.y; v[j][4 * q + 2] = x.z; v[j][4 * q + 3] = x.w;
+            }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+              const int i = (k0 + 2 * j) * 8 + u;
+              v[j][u] = 0.f;
+              const long long nd = i < K1 ? node[i].code : -1;
+              if (active && nd >= 0 && !(nd & 1)) v[j][u] = __ldg(R + (nd >> 2) * n_vec + col);
+            }
+        }
         // the patch of task it - 1 is read once its GEMM1 is done
         if (k0 == half && it > 0) ok = __all_sync(~0u, mbar_wait_timed(bar_g1, (it - 1) & 1));
         tc_fence_after();
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           if (k0 + 2 * j >= K1 / 8) continue;
+          if constexpr (WIDE) {   // to lane = column
+            __syncwarp();
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+              *reinterpret_cast<float4*>(stage + (4 * q + wj) * kStageRow + wc) =
+                  make_float4(v[j][4 * q], v[j][4 * q + 1], v[j][4 * q + 2], v[j][4 * q + 3]);
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[j][u] = stage[u * kStageRow + (t & 31)];
+          }
 #pragma unroll
           for (int u = 0; u < 8; ++u) ss += v[j][u] * v[j][u];
           tmem_st4(lane + kTmPatch + (k0 + 2 * j) * 4,
@@ -306,6 +342,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_precond_kernel(const MlpAr
     for (int task = blockIdx.x; task < n_tasks; task += gridDim.x, ++it) {
       const int buf = it & 1;
       const int col = (task % n_cb) * kTile + row;
+      const int col4 = (task % n_cb) * kTile + (warp & 3) * 32 + wc;
       const bool active = col < n_vec;
       ok = __all_sync(~0u, mbar_wait_timed(bar_g1, it & 1));
       tc_fence_after();
@@ -343,8 +380,47 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_precond_kernel(const MlpAr
         tc_fence_after();
         const int end = K1 - 128 * j < 128 ? K1 - 128 * j : 128;
         for (int c0 = half * 32; ok && c0 < end; c0 += 64) {
-          float d[32], zold[32];
+          float d[32];
           tmem_ld32(lane + (j & 1 ? kTmAcc1 : kTmAcc0) + c0, d);
+          if constexpr (WIDE) {
+            float4 zold[8];
+#pragma unroll
+            for (int g = 0; g < 8; ++g) {   // nodes c0 + 4 g + wj: r for a first colour, z otherwise
+              const int i = 128 * j + c0 + 4 * g + wj;
+              const long long nd = i < K1 ? node[i].code : -1;
+              const float* src = nd & 2 ? R : Z;
+              zold[g] = make_float4(0.f, 0.f, 0.f, 0.f);
+              if (col4 < n_vec && nd >= 0 && (nd & 3) != 1)
+                zold[g] = *reinterpret_cast<const float4*>(src + (nd >> 2) * n_vec + col4);
+            }
+#pragma unroll
+            for (int g8 = 0; g8 < 4; ++g8) {
+              __syncwarp();
+#pragma unroll
+              for (int u = 0; u < 8; ++u) {
+                const int i = 128 * j + c0 + 8 * g8 + u;
+                stage[u * kStageRow + (t & 31)] = (d[8 * g8 + u] + sh.b2[i < K1 ? i : 0]) * s;
+              }
+              __syncwarp();
+#pragma unroll
+              for (int q = 0; q < 2; ++q) {
+                const int g = 2 * g8 + q, i = 128 * j + c0 + 4 * g + wj;
+                const float4 y = *reinterpret_cast<const float4*>(stage + (4 * q + wj) * kStageRow + wc);
+                const MlpNode nd = node[i < K1 ? i : 0];
+                float4 z;   // D^-1 r, or z as it is
+                z.x = __fmul_rn(zold[g].x, nd.d); z.y = __fmul_rn(zold[g].y, nd.d);
+                z.z = __fmul_rn(zold[g].z, nd.d); z.w = __fmul_rn(zold[g].w, nd.d);
+                if (!(nd.code & 1)) {
+                  z.x = __fmaf_rn(y.x, nd.w, z.x); z.y = __fmaf_rn(y.y, nd.w, z.y);
+                  z.z = __fmaf_rn(y.z, nd.w, z.z); z.w = __fmaf_rn(y.w, nd.w, z.w);
+                }
+                if (col4 < n_vec && i < a.n3 && (nd.code & 3) != 1)
+                  *reinterpret_cast<float4*>(Z + (nd.code >> 2) * n_vec + col4) = z;
+              }
+            }
+            continue;
+          }
+          float zold[32];
           if (!active) continue;
           // all 32 reads (r for a first colour, z otherwise) are issued before
           // anything uses them or the first store
@@ -881,7 +957,10 @@ fe_status precond_apply_f32(fe_ctx* c, const float* r, float* z, int nv, cudaStr
   cudaError_t e = solver_workspace(c, 1);
   if (e != cudaSuccess) return from_cuda(e);
   const size_t smem = mlp_smem_bytes(L->K1);
-  e = ensure_dyn_smem(reinterpret_cast<const void*>(mlp_precond_kernel), smem);
+  // four columns per access where rows and blocks are aligned to them
+  const bool wide = nv % 4 == 0 && ((reinterpret_cast<uintptr_t>(r) | reinterpret_cast<uintptr_t>(z)) & 15) == 0;
+  auto kern = wide ? mlp_precond_kernel<true> : mlp_precond_kernel<false>;
+  e = ensure_dyn_smem(reinterpret_cast<const void*>(kern), smem);
   int dev = 0, sms = 0;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -894,7 +973,7 @@ fe_status precond_apply_f32(fe_ctx* c, const float* r, float* z, int nv, cudaStr
     if (nc == 0) continue;
     const long long tasks = (long long)nc * n_cb;
     if (tasks > 0x7fffffffLL) return from_cuda(cudaErrorInvalidConfiguration);
-    e = launch_kernel(mlp_precond_kernel, (size_t)std::min<long long>(tasks, sms), dim3(kMlpThreads), smem, s, overlap, a,
+    e = launch_kernel(kern, (size_t)std::min<long long>(tasks, sms), dim3(kMlpThreads), smem, s, overlap, a,
                       c->mdev, c->d_cells + c->colors.offset[k], (int)tasks, r, c->ws.dinv32, z, nv, n_cb, c->d_status);
     if (e != cudaSuccess) return from_cuda(e);
     overlap = true;
