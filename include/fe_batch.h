@@ -6,7 +6,7 @@
  * this call extends that to a batch of independent operators of different
  * size, degree and block width.  One persistent kernel takes work items
  * (problem, cell colour, range of cells, vector block) from a queue ordered
- * by colour phase; an item of colour k waits (bounded) until its problem's
+ * by each problem's progress through its colours; an item of colour k waits (bounded) until its problem's
  * colour k-1 items are done, so assembly stays conflict-free and every Y is
  * bitwise the one fe_apply produces.  The kernel and the reset of its queue
  * are captured once in a CUDA graph; each fe_batch_apply replays it.
@@ -39,9 +39,10 @@ typedef struct {
  * (FP64 data, double-float arithmetic) or FE_FP32.  Every work item runs the
  * cell body of the mode's default per-colour kernel, so results equal
  * fe_apply's bit for bit.  FE_FP64 runs one persistent kernel over all
- * problems; FE_DF64 and FE_FP32 run one persistent kernel per degree (its
- * tables as kernel parameters, its own queue) as parallel branches of the
- * graph.  All problems of one degree must use the same quadrature rule.  With autotune != 0 the vectors per work item of
+ * problems; FE_DF64 and FE_FP32 run one persistent kernel per group of
+ * problems of one degree and one aspect of their cells (the group's tables as
+ * kernel parameters, its own queue) as parallel branches of the graph.  All
+ * problems of one degree must use the same quadrature rule.  With autotune != 0 the vectors per work item of
  * every (degree, block-width bucket) are chosen by timing the candidates on
  * an 8^3 periodic proxy mesh (at most 64 vectors); otherwise a fixed rule is
  * used.  The contexts must outlive the batch.  Synchronous. */

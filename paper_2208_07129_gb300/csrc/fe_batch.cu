@@ -2,8 +2,8 @@
 // block widths) applied by ONE persistent kernel, launched from a CUDA graph.
 //
 // Work items are (problem, colour, range of cells of that colour, vector
-// block).  The queue is ordered by colour phase first (all problems' colour-0
-// items, then colour 1, ...), so an item of colour k > 0 of problem i only has
+// block).  The queue is ordered by each problem's progress through its
+// colours, so an item of colour k > 0 of problem i only has
 // to wait until every colour k-1 item of problem i is done; those were taken
 // from the queue earlier by running CTAs, so the wait always ends (and it is
 // bounded besides: a CTA that gives up records FE_ETIMEOUT).  Within a colour
@@ -409,17 +409,29 @@ fe_status build_batch(fe_batch* b, int autotune_on) {
   b->group_grid.assign(groups, 0);
   b->side.assign(groups, nullptr);
   b->join.assign(groups, nullptr);
-  // work items, phase-major within each group
+  // work items of each group, in the order of each problem's own progress:
+  // colour k of a problem of n colours stands at (k + 1/2) / n.  A problem's
+  // colours stay in order (an item only ever waits for items before it), and
+  // the 27-colour problems, whose phases are small and wait on each other, run
+  // spread over the whole batch; with all first colours first, then all
+  // second ones, their last phases were left for the end with an idle GPU
+  // (six problems of 5..20 cells: 17.9 -> 16.9 ms).
   std::vector<WorkItem> items;
   int phases = 0;
   for (int g = 0; g < groups; ++g) {
-  b->item_begin.push_back((int)items.size());
-  for (int k = 0; k < kMaxColors; ++k) {
-    bool any = false;
+    b->item_begin.push_back((int)items.size());
+    std::vector<std::pair<double, std::pair<int, int>>> order;   // progress, (problem, colour)
     for (int i = 0; i < n; ++i) {
-      fe_ctx* c = b->ctxs[i];
-      if (b->group_of[i] != g || k >= c->colors.n_colors) continue;
-      any = true;
+      const int nc = b->ctxs[i]->colors.n_colors;
+      if (b->group_of[i] != g) continue;
+      phases = std::max(phases, nc);
+      for (int k = 0; k < nc; ++k) order.push_back({(k + 0.5) / nc, {i, k}});
+    }
+    std::stable_sort(order.begin(), order.end(),
+                     [](const auto& x, const auto& y) { return x.first < y.first; });
+    for (const auto& o : order) {
+      const int i = o.second.first, k = o.second.second;
+      const fe_ctx* c = b->ctxs[i];
       const int c0 = c->colors.offset[k], c1 = c->colors.offset[k + 1];
       const BatchProblemDev<T>& P = hp[i];
       // cells per item: keep >= ~8 items per SM over the whole batch
@@ -433,8 +445,6 @@ fe_status build_batch(fe_batch* b, int autotune_on) {
           need[(size_t)i * kMaxColors + k]++;
         }
     }
-    if (any) phases = std::max(phases, k + 1);
-  }
   }
   b->item_begin.push_back((int)items.size());
   b->n_items = (int)items.size();
