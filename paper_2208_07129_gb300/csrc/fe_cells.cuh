@@ -15,6 +15,7 @@
 #pragma once
 
 #include <algorithm>
+#include <type_traits>
 
 #include "fe_arith.cuh"
 #include "fe_dispatch.cuh"
@@ -245,6 +246,13 @@ template <typename V>
 __host__ __device__ inline bool vec_ok(const void* X, const void* Y, int n_vec) {
   constexpr size_t bytes = sizeof(typename Arith<V>::D) * Arith<V>::W;
   return n_vec % Arith<V>::W == 0 && reinterpret_cast<size_t>(X) % bytes == 0 && reinterpret_cast<size_t>(Y) % bytes == 0;
+}
+
+// Scratch of a small mesh's product on this stream, or null: colour-ordered launches.
+template <typename V>
+void* small_scratch(const fe_ctx* c, cudaStream_t s) {
+  if constexpr (std::is_same<V, ff>::value) return c->small_df_scratch(s);
+  return c->d_small;
 }
 
 // CTA of a small mesh: every line of a pass has a thread, and B vector groups

@@ -320,14 +320,15 @@ cudaError_t launch_general(const fe_ctx* c, const typename Arith<V>::D* X, typen
   const bool vec = vec_ok<V>(X, Y, n_vec);
   const auto tab = make_generaltables<typename Arith<V>::C, NP, NQ>(c);
   if constexpr (!SC) {   // small meshes, as in launch_box
-    if (c->d_small && (size_t)n_vec * NP * NP * NP * c->n_cells * sizeof(D) <= c->small_bytes) {
+    const bool fits = (size_t)n_vec * NP * NP * NP * c->n_cells * sizeof(D) <= c->small_bytes;
+    if (void* scratch = fits ? small_scratch<V>(c, s) : nullptr) {
       auto lk = cell_apply_general_local_kernel<V, NP, NQ>;
       int lanes = 1;
       size_t lsm = 0;
       cudaError_t e = small_shape<V, NQ, 3>(c->n_cells, n_vec, &lanes, &lsm);
       if (e == cudaSuccess) e = ensure_dyn_smem(reinterpret_cast<const void*>(lk), lsm);
       if (e != cudaSuccess) return e;
-      D* Wk = static_cast<D*>(c->d_small);
+      D* Wk = static_cast<D*>(scratch);
       const int blocks = (n_vec + lanes * W - 1) / (lanes * W);
       e = launch_kernel(lk, c->n_cells * (size_t)blocks, dim3(lanes, NQ * NQ), lsm, s, false, tab, c->mdev, geo, n_vec,
                         blocks, vec, X, Wk);

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <atomic>
 #include <cstdint>
 #include <vector>
 
@@ -44,8 +45,8 @@ struct Tables {
 // Geometry of the quadrature-point operation.  With weights folded into the
 // tables:  G_sd = mu det J (J^-1 J^-T)_sd   and   c = det J V.
 // Affine cells (axis-aligned boxes): one G per cell (cellG[e*6 + k],
-// k = 00,01,02,11,12,22), diagonal: the even-odd and double-float bodies
-// read only k = 00, 11, 22.
+// k = 00,01,02,11,12,22), diagonal; the box kernel reads only k = 22 (the
+// ratios to the others are part of its tables).
 // General (trilinear) cells: ptG[(e*6 + k) * nq3 + Q].  Always ptC[e*nq3 + Q].
 template <typename T>
 struct Geom {
@@ -175,8 +176,8 @@ struct fe_ctx {
   fe::LineTile tile64() const { return set64 ? fe::LineTile{vb64, nty64} : fe::LineTile{0, 0}; }
   fe::LineTile tile32() const { return set32 ? fe::LineTile{vb32, nty32} : fe::LineTile{0, 0}; }
   fe::LineTile tiledf() const { return setdf ? fe::LineTile{vbdf, ntydf} : fe::LineTile{0, 0}; }
-  int fp32_variant = 0;   // 0 / 1: line kernel, 2: register-plane kernel, 3: even-odd line kernel
-  int fp64_variant = 0;   // 0: even-odd line kernel, 1: plain line kernel
+  int fp32_variant = 0;   // 0 / 1: line kernel, 2: register-plane kernel, 3: box / trilinear kernel
+  int fp64_variant = 0;   // 0: box / trilinear kernel, 1: plain line kernel
   int tc_variant = 0;     // FE_TF32 / FE_BF16 / FE_BF16S: 0 tcgen05 kernel (where built) with TMA boxes where
                           // the blocks allow, 1 warp-MMA kernel (not FE_BF16S), 2 tcgen05 with thread loads/stores
   // B operands of the tcgen05 kernel's six passes (TF32, BF16), built at setup
@@ -191,6 +192,24 @@ struct fe_ctx {
   // colour; allocated at setup
   void* d_small = nullptr;
   size_t small_bytes = 0;
+  // the same for double-float products, which have a scratch of their own and
+  // use it on one stream only (the first that asks): a product on another
+  // stream, or one being captured, takes the colour-ordered launches, so small
+  // double-float products of a context need no order between streams
+  void* d_small_df = nullptr;
+  mutable std::atomic<intptr_t> small_df_stream{-1};
+  void* small_df_scratch(cudaStream_t s) const {
+    if (!d_small_df || s == cudaStreamPerThread) return nullptr;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+      cudaGetLastError();   // the legacy stream while another thread captures
+      return nullptr;
+    }
+    if (cap != cudaStreamCaptureStatusNone) return nullptr;
+    intptr_t owner = -1;
+    const intptr_t me = reinterpret_cast<intptr_t>(s);
+    return small_df_stream.compare_exchange_strong(owner, me) || owner == me ? d_small_df : nullptr;
+  }
 };
 
 namespace fe {

@@ -422,6 +422,7 @@ extern "C" fe_status fe_setup(const fe_mesh_desc* mesh, int p, const fe_quad_des
   if (err == cudaSuccess && E * (size_t)c->np * c->np * c->np <= kSmallSlots) {
     c->small_bytes = E * (size_t)c->np * c->np * c->np * 64 * sizeof(double);
     err = cudaMalloc(&c->d_small, c->small_bytes);
+    if (err == cudaSuccess) err = cudaMalloc(&c->d_small_df, c->small_bytes);
   }
   if (err != cudaSuccess) { fe_destroy(c); return from_cuda(err); }
   *out = c;
@@ -435,6 +436,7 @@ extern "C" void fe_destroy(fe_ctx* c) {
   cudaFree(c->d_cellGff); cudaFree(c->d_ptGff); cudaFree(c->d_ptCff);
   cudaFree(c->d_status); cudaFree(c->d_stage);
   cudaFree(c->d_tcimg[0]); cudaFree(c->d_tcimg[1]); cudaFree(c->d_tcmask); cudaFree(c->d_tcq); cudaFree(c->d_small);
+  cudaFree(c->d_small_df);
   if (c->copy_in) cudaStreamDestroy(c->copy_in);
   if (c->copy_out) cudaStreamDestroy(c->copy_out);
   for (cudaEvent_t ev : {c->ev_start, c->ev_in[0], c->ev_in[1], c->ev_comp[0], c->ev_comp[1], c->ev_out[0], c->ev_out[1]})
