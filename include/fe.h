@@ -173,8 +173,9 @@ fe_mode fe_get_mode(const fe_ctx* ctx);
 /* Y = A X for n_vec >= 0 vectors (Algorithm 2 per cell, batched over cells and
  * vector blocks as in Algorithm 4, assembled by cell colours: no two cells of
  * a colour share a node and colours run in order, so every node's sum is
- * formed in a fixed order and results are deterministic; the tcgen05 kernel's
- * TMA path zeroes Y and adds each cell's result box with a bulk reduce).
+ * formed in a fixed order and results are deterministic; a colour's launch may
+ * start while the one before it finishes, but touches Y only after it; the
+ * tcgen05 kernel's TMA path zeroes Y and adds each cell's result box with a bulk reduce).
  * X, Y: device, num_dofs x n_vec, dtype of the current mode, X != Y (no
  * overlap).  Y is overwritten, never accumulated.  Asynchronous on stream.
  * On a refined mesh with hanging nodes the product first distributes X into a
@@ -185,13 +186,16 @@ fe_mode fe_get_mode(const fe_ctx* ctx);
 fe_status fe_apply(fe_ctx* ctx, const void* X, void* Y, int n_vec, void* stream);
 
 /* Launch shape of the CUDA-core cell kernels of one mode (the autotuner's
- * knob): vectors per CTA (power of two, 1..32; halved further when shared
- * memory does not hold it, and never above the padded n_vec), lines in flight
+ * knob): vectors per CTA (power of two, 1..32, at least the two that an FP32
+ * thread of variant 3 works on; halved further when shared memory does not
+ * hold it, and never above the padded n_vec), lines in flight
  * per CTA (1..256; CTAs are capped at 256 threads), and the variant
- * (FE_FP64: 0 = line kernel with even-odd contractions, 1 = plain line
- * kernel; FE_FP32: 0 or 1 = line kernel, 2 = register-plane kernel, n_q <= 8
- * only, 3 = line kernel with even-odd contractions; FE_DF64: 0, the
- * double-float even-odd line kernel).
+ * (FE_FP64: 0 = box or trilinear kernel with even-odd contractions, 1 = plain
+ * line kernel; FE_FP32: 0 or 1 = plain line kernel, 2 = register-plane kernel,
+ * n_q <= 8 only, 3 = box or trilinear kernel with even-odd contractions (the
+ * default); FE_DF64: 0, the same kernels in double-float arithmetic).  Until a
+ * tile is set the default kernels choose theirs by n_q.  Results do not depend
+ * on the tile.
  * FE_TF32 / FE_BF16 / FE_BF16S (one setting for the three): the tile is
  * fixed; variant 0 = tcgen05 kernel where built (n_p, n_q <= 8), moving each
  * cell's values with TMA boxes when X and Y are 16-byte aligned and a node's

@@ -36,8 +36,8 @@ fe_status fe_mass_gll(fe_ctx* ctx, double* m_host);
  * with the M^-1/2 scalings folded into the gather and the scatter and the
  * b X + c Y terms into the first write of each node (colour-ordered
  * assembly), so the product costs one pass over X and Y like fe_apply.
- * Mode FE_FP64 (even-odd cell kernel), FE_DF64 (FP64 data, double-float
- * arithmetic) or FE_FP32 (even-odd line kernel in FP32); the tensor-core
+ * Mode FE_FP64, FE_DF64 (FP64 data, double-float arithmetic) or FE_FP32 (the
+ * box and trilinear cell kernels); the tensor-core
  * modes return FE_EUNSUPPORTED.  X and Y must not overlap.  Y is
  * read only when c != 0 (it may be uninitialised when c == 0).  Constrained
  * rows of Y are written 0. */

@@ -1,6 +1,6 @@
-// FP32 CUDA-core instantiations: the line kernel, the line kernel with
-// even-odd contractions, or the register-plane kernel (n_q <= 8), as
-// selected with fe_set_tile.
+// FP32 CUDA-core instantiations: the box and trilinear kernels (default), the
+// plain line kernel, or the register-plane kernel (n_q <= 8), as selected
+// with fe_set_tile.
 #include "fe_dispatch.cuh"
 #include "fe_box.cuh"
 #include "fe_general.cuh"

@@ -1,4 +1,4 @@
-// FP64 CUDA-core instantiations of the fused cell kernel (even-odd by
+// FP64 CUDA-core instantiations of the cell kernels (box or trilinear by
 // default, the plain line kernel as variant 1) and of the diagonal.
 #include "fe_dispatch.cuh"
 #include "fe_box.cuh"

@@ -1,5 +1,5 @@
 // FP64 instantiations of the scaled product of the Chebyshev filter,
-// Y = a M^-1/2 A M^-1/2 X + b X + c Y (even-odd cell kernel).
+// Y = a M^-1/2 A M^-1/2 X + b X + c Y (box and trilinear kernels).
 #include "fe_dispatch.cuh"
 #include "fe_box.cuh"
 #include "fe_general.cuh"
