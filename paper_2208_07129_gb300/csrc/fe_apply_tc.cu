@@ -163,6 +163,7 @@ cudaError_t launch_tc(const fe_ctx* c, const unsigned char* img, const TIO* X, T
   if (QF && TMA && c->d_ptCtc == nullptr) return cudaErrorInvalidValue;
   const int n_vb = (n_vec + kTcVectors - 1) / kTcVectors;
   if (TMA && c->colors.n_colors > kTcQueues) return cudaErrorInvalidValue;
+  bool overlap = false;   // see launch_kernel
   for (int k = 0; k < c->colors.n_colors; ++k) {
     const int n = c->colors.offset[k + 1] - c->colors.offset[k];
     if (n == 0) continue;
@@ -171,9 +172,10 @@ cudaError_t launch_tc(const fe_ctx* c, const unsigned char* img, const TIO* X, T
     const int grid = (int)std::min<long long>((tasks + SH::SLOTS - 1) / SH::SLOTS, (long long)sms);
     a.cmask = c->d_tcmask + c->colors.offset[k];
     a.queue = c->d_tcq + k;
-    kern<<<grid, 128 * SH::SLOTS, smem, s>>>(a, c->mdev, geo, c->d_cells + c->colors.offset[k], (int)tasks, n_vec,
-                                              n_vb, X, Y, xm, ym);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    e = launch_kernel(kern, (size_t)grid, dim3(128 * SH::SLOTS), smem, s, overlap, a, c->mdev, geo,
+                      c->d_cells + c->colors.offset[k], (int)tasks, n_vec, n_vb, X, Y, xm, ym);
+    if (e != cudaSuccess) return e;
+    overlap = true;
   }
   return cudaSuccess;
 }

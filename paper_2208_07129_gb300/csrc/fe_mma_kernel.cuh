@@ -21,7 +21,7 @@
 
 #include <cuda_bf16.h>
 
-#include "fe_cell_kernel.cuh"
+#include "fe_dispatch.cuh"
 
 namespace fe {
 
@@ -252,6 +252,7 @@ __global__ void __launch_bounds__(32 * kMmaWarps) mma_apply_kernel(const Tables<
   constexpr int P = NP - 1;
   constexpr int NQ3 = NQ * NQ * NQ;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  let_next_launch_start();
   float* base = reinterpret_cast<float*>(smem_raw);
   const int warp = threadIdx.x >> 5;
   const int vb = blockIdx.x % n_vb;
@@ -370,6 +371,7 @@ __global__ void __launch_bounds__(32 * kMmaWarps) mma_apply_kernel(const Tables<
     pass<KIND, NQ, NP, false>(f, Tile{S1q.p, NQ, NQ, NP}, Tile{S0q.p, NQ, NP, NP}, 1, NQ * NP);
   }
   __syncthreads();
+  wait_for_earlier_launch();
   {  // transposed x pass of N fused with assembly
     BFrags<KIND, NQ, NP> f;
     load_bfrags(f, tab.N, true);
@@ -411,15 +413,14 @@ cudaError_t launch_mma(const fe_ctx* c, const float* X, float* Y, int n_vec, cud
   const Tables<float, NP, NQ> tab = make_tables<float, NP, NQ>(c);
   const Geom<float> geo = make_geom<float>(c);
   const int n_vb = (n_vec + kMmaVB - 1) / kMmaVB;
+  bool overlap = false;   // see launch_kernel
   for (int k = 0; k < c->colors.n_colors; ++k) {
     const int n = c->colors.offset[k + 1] - c->colors.offset[k];
     if (n == 0) continue;
-    const long long blocks = (long long)n * n_vb;
-    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    kern<<<(unsigned)blocks, 32 * kMmaWarps, smem, s>>>(tab, c->mdev, geo, c->d_cells + c->colors.offset[k], n_vec,
-                                                         n_vb, X, Y);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_kernel(kern, (size_t)n * n_vb, dim3(32 * kMmaWarps), smem, s, overlap, tab, c->mdev, geo,
+                                        c->d_cells + c->colors.offset[k], n_vec, n_vb, X, Y);
     if (e != cudaSuccess) return e;
+    overlap = true;
   }
   return cudaSuccess;
 }

@@ -42,7 +42,7 @@
 
 #include <cuda_bf16.h>
 
-#include "fe_cell_kernel.cuh"
+#include "fe_dispatch.cuh"
 #include "fe_tma.cuh"
 #include "fe_umma.cuh"
 
@@ -274,6 +274,16 @@ __device__ __forceinline__ TIO tc_zero() {
   if constexpr (sizeof(TIO) == 4) return 0.f;
   else return __ushort_as_bfloat16((unsigned short)0);
 }
+// The colours' launches overlap (see launch_kernel): BF16 32^3 p = 6 3.86 -> 3.83
+// ms, and small products, whose colours are one task's latency each, 191 -> 63 us.
+// Before a thread's first access to Y: the colours before have completed, and
+// bulk (async proxy) operations issued from here on follow their stores.
+__device__ __forceinline__ void wait_for_earlier_colour(bool& first) {
+  if (!first) return;
+  wait_for_earlier_launch();
+  asm volatile("fence.proxy.async;" ::: "memory");
+  first = false;
+}
 __device__ __forceinline__ void tc_atomic_add(float* p, float v) { atomicAdd(p, v); }
 __device__ __forceinline__ void tc_atomic_add(__nv_bfloat16* p, float v) { atomicAdd(p, __float2bfloat16_rn(v)); }
 
@@ -348,6 +358,7 @@ __global__ void __launch_bounds__(128 * TcShape<E, G, KIND>::SLOTS, 1)
     }
   }
 
+  let_next_launch_start();
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
                  "r"(SH::TMEM_COLS));
@@ -375,7 +386,7 @@ __global__ void __launch_bounds__(128 * TcShape<E, G, KIND>::SLOTS, 1)
   tc_fence_after();
   const uint32_t tmem = *tslot + (uint32_t)(slot * SH::SLOT_COLS);
   const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-  bool fail = false, load_pending = false;
+  bool fail = false, load_pending = false, first_write = true;
   uint32_t lphase = 0;
 
   // TMA kernels take their tasks from the launch's counter, one at a time
@@ -664,10 +675,12 @@ __global__ void __launch_bounds__(128 * TcShape<E, G, KIND>::SLOTS, 1)
       fence_async_smem();
       slot_sync(bar);
       if (lt == 0) {
+        wait_for_earlier_colour(first_write);
         tma_reduce_add_4d(&ymap, box, v0, cx * P, cy * P, cz * P);
         bulk_commit();
       }
     } else {
+      wait_for_earlier_colour(first_write);
 #pragma unroll 1
       for (int j = 0; j < T; ++j) {   // B-x and assembly: row (i3, b), lines i2 = G b + g, D = [g][i1]
         float d[SH::Nr(5)];
@@ -721,6 +734,7 @@ __global__ void __launch_bounds__(128 * TcShape<E, G, KIND>::SLOTS, 1)
   if constexpr (TMA) {
     if (lt == 0) bulk_wait_all();   // the reduces of this slot are complete
   }
+  wait_for_earlier_launch();   // every CTA, so that the colours complete in order
   tc_fence_before();
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tslot), "r"(SH::TMEM_COLS));
