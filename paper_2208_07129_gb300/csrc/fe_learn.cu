@@ -161,6 +161,18 @@ __host__ __device__ constexpr size_t mlp_smem_bytes(int K1) {
          (size_t)kMlpThreads / 32 * 8 * kStageRow * sizeof(float);
 }
 
+// What a launch asks for: always more than half of an SM's 228 KB, so that one
+// CTA is on an SM at a time whatever the degree (the tables of p <= 3 take 36 to
+// 60 KB) and however many registers the compiler takes.  Every CTA allocates
+// all of the SM's tensor memory; with two of them on an SM, one of a later
+// colour could hold it while it waits for an earlier colour's CTA that waits
+// for the memory.
+constexpr size_t kSmSharedBytes = 228 * 1024;
+__host__ __device__ constexpr size_t mlp_smem_request(int K1) {
+  return mlp_smem_bytes(K1) > kSmSharedBytes / 2 ? mlp_smem_bytes(K1) : kSmSharedBytes / 2 + 1024;
+}
+static_assert(2 * mlp_smem_request(16) > kSmSharedBytes, "two CTAs must not fit on one SM");
+
 template <bool WIDE>
 __global__ void __launch_bounds__(kMlpThreads, 1) mlp_precond_kernel(const MlpArgs a, const MeshDev m,
                                                                      const int* __restrict__ cells, int n_tasks,
@@ -188,7 +200,6 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_precond_kernel(const MlpAr
   const int n_chunks = (K1 + 127) / 128;
   const int P = a.np - 1;
 
-  let_next_launch_start();
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(sh.tslot)),
                  "r"(kTmemCols));
@@ -209,6 +220,9 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_precond_kernel(const MlpAr
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // not before the blocking allocation has returned: no CTA of the next colour
+  // can then take the tensor memory that this colour's still wait for
+  let_next_launch_start();
   const uint32_t tmem = *sh.tslot;
   float* stage = sh.stage + warp * 8 * kStageRow;
   const uint32_t lane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
@@ -956,7 +970,7 @@ fe_status precond_apply_f32(fe_ctx* c, const float* r, float* z, int nv, cudaStr
   if (L->K1 > 352) return FE_EUNSUPPORTED;
   cudaError_t e = solver_workspace(c, 1);
   if (e != cudaSuccess) return from_cuda(e);
-  const size_t smem = mlp_smem_bytes(L->K1);
+  const size_t smem = mlp_smem_request(L->K1);
   // four columns per access where rows and blocks are aligned to them
   const bool wide = nv % 4 == 0 && ((reinterpret_cast<uintptr_t>(r) | reinterpret_cast<uintptr_t>(z)) & 15) == 0;
   auto kern = wide ? mlp_precond_kernel<true> : mlp_precond_kernel<false>;
