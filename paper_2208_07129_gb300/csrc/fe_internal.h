@@ -256,7 +256,7 @@ void free_refined(fe_ctx* c);
 void build_gll_mass(fe_ctx* c);
 void free_eig(fe_ctx* c);
 // Solver workspace and the learned preconditioner (fe_solve.cu / fe_learn.cu).
-cudaError_t solver_workspace(fe_ctx* c, int nv);
+cudaError_t solver_workspace(fe_ctx* c, int nv, cudaStream_t s);
 void free_solver_workspace(fe_ctx* c);
 bool learned_ready(const fe_ctx* c, int nv);
 fe_status learned_precond_apply(fe_ctx* c, const void* r, void* z, int nv, bool fp64, cudaStream_t s);

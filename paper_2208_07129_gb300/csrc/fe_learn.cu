@@ -968,7 +968,7 @@ fe_status precond_apply_f32(fe_ctx* c, const float* r, float* z, int nv, cudaStr
   LearnedPrecond* L = c->learned;
   if (!L || !L->images_valid) return FE_EINVAL;
   if (L->K1 > 352) return FE_EUNSUPPORTED;
-  cudaError_t e = solver_workspace(c, 1);
+  cudaError_t e = solver_workspace(c, 1, s);
   if (e != cudaSuccess) return from_cuda(e);
   const size_t smem = mlp_smem_request(L->K1);
   // four columns per access where rows and blocks are aligned to them
@@ -1443,7 +1443,7 @@ extern "C" fe_status fe_energy_gradients(fe_ctx* c, const float* R, const float*
   LearnedPrecond* L = c->learned;
   const int n3 = L->n3;
   const size_t tot = c->n_dofs * (size_t)n_vec, rows = c->n_cells * (size_t)n_vec;
-  cudaError_t e = solver_workspace(c, n_vec);   // the Jacobi diagonal of z = D^-1 r + ...
+  cudaError_t e = solver_workspace(c, n_vec, s);   // the Jacobi diagonal of z = D^-1 r + ...
   if (e != cudaSuccess) return from_cuda(e);
   std::vector<int> hcells(c->n_cells);
   for (size_t k = 0; k < c->n_cells; ++k) hcells[k] = (int)k;
@@ -1490,7 +1490,7 @@ extern "C" fe_status fe_precond_train(fe_ctx* c, const fe_train_desc* d, fe_trai
   LearnedPrecond* L = c->learned;
   const int nv = d->n_rhs, n3 = L->n3;
   const size_t n = c->n_dofs, tot = n * nv;
-  cudaError_t e = solver_workspace(c, nv);
+  cudaError_t e = solver_workspace(c, nv, s);
   if (e != cudaSuccess) return from_cuda(e);
 
   // right-hand sides ~ N(0,1), Dirichlet rows zero (host PRNG, seeded)

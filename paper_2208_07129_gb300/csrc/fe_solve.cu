@@ -584,7 +584,7 @@ cudaError_t grow(T** p, size_t* cap, size_t n) {
 
 namespace fe {
 
-cudaError_t solver_workspace(fe_ctx* c, int nv) {
+cudaError_t solver_workspace(fe_ctx* c, int nv, cudaStream_t s) {
   SolveWs& w = c->ws;
   const size_t n = c->n_dofs, tot = n * (size_t)nv;
   cudaError_t e = cudaSuccess;
@@ -595,7 +595,14 @@ cudaError_t solver_workspace(fe_ctx* c, int nv) {
   if (e == cudaSuccess) e = grow(&w.active, &w.cap_active, (size_t)nv);
   if (e == cudaSuccess && w.cap_ticket < (size_t)nv) {
     e = grow(&w.ticket, &w.cap_ticket, (size_t)nv);
-    if (e == cudaSuccess) e = cudaMemset(w.ticket, 0, (size_t)nv * sizeof(int));
+    // zeroed on the caller's stream (one that does not wait for the legacy
+    // stream must not start counting first), and before the call goes on, since
+    // the next caller may come on another stream
+    if (e == cudaSuccess) {
+      e = cudaMemsetAsync(w.ticket, 0, (size_t)nv * sizeof(int), s);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      if (e != cudaSuccess) w.cap_ticket = 0;
+    }
   }
   if (e == cudaSuccess && !w.dinv64) {
     e = cudaMalloc(&w.dinv64, n * sizeof(double));
@@ -807,7 +814,7 @@ extern "C" fe_status fe_solve(fe_ctx* c, const double* B, double* X, int nv, dou
     return FE_EINVAL;
   if (precond == FE_PRECOND_LEARNED && !learned_ready(c, nv)) return FE_EINVAL;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  cudaError_t e = solver_workspace(c, nv);
+  cudaError_t e = solver_workspace(c, nv, s);
   if (e != cudaSuccess) return from_cuda(e);
   SolveWs& w = c->ws;
   const size_t n = c->n_dofs, tot = n * (size_t)nv;
