@@ -182,7 +182,17 @@ fe_mode fe_get_mode(const fe_ctx* ctx);
  * context-owned device block of X's size (X with the slave rows filled in);
  * the first call with a given or larger n_vec allocates that block
  * (cudaMalloc, which synchronises the device), later calls reuse it.
- * fe_apply_host_noalloc takes the block from its fixed array instead. */
+ * fe_apply_host_noalloc takes the block from its fixed array instead.
+ * Order: products of one context on one stream may come from several host
+ * threads.  In FE_FP64, FE_DF64, FE_FP32 and FE_TF32X3 on structured meshes
+ * they may also run on several streams and as replays of captured graphs at
+ * the same time (small meshes keep a block of scratch for products outside
+ * captures and one each for three pairs of capture and stream, given back with
+ * the graph; a product that finds none free runs colour by colour, with the
+ * same bits; a graph instantiated twice must not run beside itself).  In
+ * FE_TF32, FE_BF16 and FE_BF16S (task counters in the context) and on refined
+ * meshes with hanging nodes (the block above) products on different streams
+ * have to be ordered by the caller. */
 fe_status fe_apply(fe_ctx* ctx, const void* X, void* Y, int n_vec, void* stream);
 
 /* Launch shape of the CUDA-core cell kernels of one mode (the autotuner's

@@ -28,6 +28,7 @@ extern "C" fe_status fe_apply(fe_ctx* c, const void* X, void* Y, int n_vec, void
   if (overlaps(X, Y, bytes)) return FE_EINVAL;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaError_t e;
+  std::lock_guard<std::mutex> hold(c->order);
   if (c->refined) {
     if (c->mode != FE_FP64 && c->mode != FE_DF64 && c->mode != FE_FP32) return FE_EUNSUPPORTED;
     return from_cuda(apply_refined(c, X, Y, n_vec, s));

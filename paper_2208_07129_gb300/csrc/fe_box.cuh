@@ -267,8 +267,8 @@ cudaError_t launch_box(const fe_ctx* c, const typename Arith<V>::D* X, typename 
   if constexpr (!SC && !MAP) {
     // Small meshes (scratch allocated at setup): one launch over all cells
     // writing each cell's result to the scratch, then one gather in colour order.
-    const bool fits = (size_t)n_vec * NP * NP * NP * c->n_cells * sizeof(D) <= c->small_bytes;
-    if (void* scratch = fits ? small_scratch<V>(c, s) : nullptr) {
+    const bool fits = (size_t)n_vec * NP * NP * NP * c->n_cells * sizeof(D) <= c->small.bytes();
+    if (void* scratch = fits ? c->small.block(s) : nullptr) {
       auto lk = cell_apply_box_local_kernel<V, NP, NQ>;
       int lanes = 1;
       size_t lsm = 0;
@@ -279,10 +279,13 @@ cudaError_t launch_box(const fe_ctx* c, const typename Arith<V>::D* X, typename 
       const int blocks = (n_vec + lanes * W - 1) / (lanes * W);
       e = launch_kernel(lk, c->n_cells * (size_t)blocks, dim3(lanes, NQ * NQ), lsm, s, false, tab, c->mdev, geo, n_vec,
                         blocks, vec, X, Wk);
-      if (e != cudaSuccess) return e;
-      const size_t tot = c->n_dofs * (size_t)n_vec;
-      return launch_kernel(assemble_local_kernel<D, NP>, std::min<size_t>((tot + 255) / 256, 152 * 8), dim3(256), 0, s,
-                           true, c->mdev, Wk, Y, c->n_dofs, n_vec);
+      if (e == cudaSuccess) {
+        const size_t tot = c->n_dofs * (size_t)n_vec;
+        e = launch_kernel(assemble_local_kernel<D, NP>, std::min<size_t>((tot + 255) / 256, 152 * 8), dim3(256), 0, s,
+                          true, c->mdev, Wk, Y, c->n_dofs, n_vec);
+      }
+      const cudaError_t e2 = c->small.enqueued(s);
+      return e != cudaSuccess ? e : e2;
     }
   }
   auto kern = cell_apply_box_kernel<V, NP, NQ, SC, MAP>;

@@ -248,13 +248,6 @@ __host__ __device__ inline bool vec_ok(const void* X, const void* Y, int n_vec) 
   return n_vec % Arith<V>::W == 0 && reinterpret_cast<size_t>(X) % bytes == 0 && reinterpret_cast<size_t>(Y) % bytes == 0;
 }
 
-// Scratch of a small mesh's product on this stream, or null: colour-ordered launches.
-template <typename V>
-void* small_scratch(const fe_ctx* c, cudaStream_t s) {
-  if constexpr (std::is_same<V, ff>::value) return c->small_df_scratch(s);
-  return c->d_small;
-}
-
 // CTA of a small mesh: every line of a pass has a thread, and B vector groups
 // share a CTA, B chosen so that the fullest SM has the fewest warps: with few
 // cells a CTA's time is its passes' latency, and partly filled warps cost the

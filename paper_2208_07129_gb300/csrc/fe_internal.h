@@ -2,18 +2,19 @@
 #pragma once
 
 #include <cuda_runtime.h>
-#include <atomic>
 #include <cstdint>
+#include <mutex>
 #include <vector>
 
 #include "../../include/fe.h"
 #include "fe_arith.cuh"
 #include "fe_ff.cuh"
+#include "fe_small.h"
 
 namespace fe {
 
 constexpr int kMaxP = 8;
-constexpr size_t kSmallSlots = 16384;   // cells x n_p^3 of a "small" mesh (see fe_ctx::d_small)
+constexpr size_t kSmallSlots = 16384;   // cells x n_p^3 of a "small" mesh (see fe_ctx::small)
 constexpr int kMaxNQ = kMaxP + 3;
 
 // Entries of the explicit cell -> DoF map of refined meshes: the DoF index in
@@ -190,26 +191,11 @@ struct fe_ctx {
   // small meshes (E n_p^3 <= kSmallSlots): per-cell result scratch for up to
   // 64 FP64 vectors, so that fe_apply runs as two launches instead of one per
   // colour; allocated at setup
-  void* d_small = nullptr;
-  size_t small_bytes = 0;
-  // the same for double-float products, which have a scratch of their own and
-  // use it on one stream only (the first that asks): a product on another
-  // stream, or one being captured, takes the colour-ordered launches, so small
-  // double-float products of a context need no order between streams
-  void* d_small_df = nullptr;
-  mutable std::atomic<intptr_t> small_df_stream{-1};
-  void* small_df_scratch(cudaStream_t s) const {
-    if (!d_small_df || s == cudaStreamPerThread) return nullptr;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
-      cudaGetLastError();   // the legacy stream while another thread captures
-      return nullptr;
-    }
-    if (cap != cudaStreamCaptureStatusNone) return nullptr;
-    intptr_t owner = -1;
-    const intptr_t me = reinterpret_cast<intptr_t>(s);
-    return small_df_stream.compare_exchange_strong(owner, me) || owner == me ? d_small_df : nullptr;
-  }
+  mutable fe::SmallScratch small;
+  // held by fe_apply while it enqueues a product: a product's launches share
+  // scratch and counters of the context, and those of two host threads on one
+  // stream must not interleave
+  std::mutex order;
 };
 
 namespace fe {
