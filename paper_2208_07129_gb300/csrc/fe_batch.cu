@@ -569,14 +569,16 @@ extern "C" fe_status fe_batch_create(fe_ctx* const* ctxs, int n, const int* n_ve
 extern "C" fe_status fe_batch_apply(fe_batch* b, const void* const* X, void* const* Y, void* stream) {
   if (!b || !X || !Y) return FE_EINVAL;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  for (int i = 0; i < b->n; ++i) {
+  for (int i = 0; i < b->n; ++i)
     if (!X[i] || !Y[i] || X[i] == Y[i]) return FE_EINVAL;
+  // the copy of the last call may still be reading the staging table
+  cudaError_t e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) return from_cuda(e);
+  for (int i = 0; i < b->n; ++i) {
     b->h_ptrs[2 * i] = X[i];
     b->h_ptrs[2 * i + 1] = Y[i];
   }
-  // the table is read by the kernel of this launch; wait for the previous use of the staging buffer
-  cudaError_t e = cudaStreamSynchronize(s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_ptrs, b->h_ptrs, 2 * b->n * sizeof(void*), cudaMemcpyHostToDevice, s);
+  e = cudaMemcpyAsync(b->d_ptrs, b->h_ptrs, 2 * b->n * sizeof(void*), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaGraphLaunch(b->exec, s);
   return from_cuda(e);
 }
