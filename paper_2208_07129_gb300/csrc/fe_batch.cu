@@ -33,7 +33,7 @@ namespace fe {
 
 constexpr int kBatchThreads = 128;
 constexpr int kMaxColors = 27;
-constexpr int kTabImage = 256;   // elements of a BoxTables<T, NP, NQ> image (245 at p = 8, n_q = 10)
+constexpr int kTabImage = 208;   // elements of a BoxTables<T, NP, NQ> image (202 at p = 8, n_q = 10)
 
 template <typename T>
 struct BatchProblemDev {

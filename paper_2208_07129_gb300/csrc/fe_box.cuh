@@ -7,17 +7,28 @@
 //   D~_x^T g00 D~_x + D~_y^T g11 D~_y + D~_z^T g22 D~_z,   and   D~^T D~ = K
 // is one symmetric n_q x n_q matrix: three 1D passes with K take the place of
 // the six passes with D~ and D~^T of trilinear cells (fe_general.cuh), and
-// nothing but the values t = N u has to be kept besides their image s.  K is
-// formed in FP64 on the host; the cell's one factor g22 multiplies at the end
-// (g00 / g22 and g11 / g22 are the same for every cell of a mesh and are part
-// of the x and y tables).
+// nothing but the values t = N u has to be kept besides their image s.  The
+// cell's one factor g22 multiplies at the end (g00 / g22 and g11 / g22 are the
+// same for every cell of a mesh and are part of the tables).
 //
 // Each 1D matrix is (skew-)centrosymmetric, so it splits into an even and an
 // odd half (see fe_cells.cuh).  Here the halves stay apart between passes:
 // a direction's values are kept as (even, odd) parts from N's pass until the
 // pass that needs point values, so K works on them without sums before or
-// after.  For p = 6, n_q = 8 a cell and vector take 22.5 K operations against
-// 36.2 K for the D~ form.
+// after.
+//
+// K is applied in factors.  As one rounded matrix it would no longer annihilate
+// the constant, and the energy x.(A x) that a solver or a filter takes from the
+// product would have a first-order error of eps |K| there (FP32, 12^3 cells, p =
+// 6: 4e-4 of the energy of a constant, 6e-6 of one period's); with D~ the energy
+// is |D~ t|^2 and the rounding of a table enters it squared.  So each half is
+// kept as L^T d L, L unit lower triangular, with the rank the half has: the
+// energy is a sum of products of (L t)_k with d_k (L t)_k, both of which are
+// small where t is smooth.  Rows start at the centre of the rule and go out, and
+// the centre itself has none.  FP32 energies are then as accurate as the D~
+// form's (1.2e-7 and 1.1e-7).  L and d L^T take R (R + 1) / 2 products each, less
+// L's unit diagonal: one operation less than the matrix.  For p = 6, n_q = 8 a
+// cell and vector take 22.1 K operations against 36.2 K for the D~ form.
 //
 // Seven passes over 1D lines, each thread one line (W vectors of it) in
 // registers, in place on two shared tiles t and s of n_q^3 values per vector:
@@ -31,26 +42,87 @@
 // the distance of two groups is chosen so that no pass meets a bank conflict.
 //
 // What bounds it, and what it measured (32^3 periodic, p = 6, n_q = 8, 64
-// vectors; the D~ form before): FP64 148.0 -> 89.9 ms, the FP64 pipe (22.5 K
-// operations at 0.595 T/s are 79 ms); double-float 38.9 -> 20.9 ms, the issue
-// of FP32 instructions.  FP32, 24^3, 128 vectors: 6.92 -> 2.99 ms, shared
+// vectors; the D~ form before): FP64 148.0 -> 89.3 ms, the FP64 pipe (22.1 K
+// operations at 0.595 T/s are 78 ms); double-float 38.9 -> 21.9 ms, the issue
+// of FP32 instructions.  FP32, 24^3, 128 vectors: 6.92 -> 3.03 ms, shared
 // memory (7.5 K values per cell and vector, 1.2 ms) and the barriers between
-// the passes.
+// the passes.  With K as one matrix the three were 89.9, 21.4 and 3.00 ms; the
+// 12^3 p = 6 solve with FP32 inner iterations took 156 ms with it and takes 148.
 #pragma once
 
 #include "fe_cells.cuh"
 
 namespace fe {
 
+// K = L^T d L by halves of R rows: R = RE for the even half, which has one part
+// more, the centre; R = RO for the odd half.  L, the same for every direction:
+// row k has e[k (k-1)/2 + i] for the parts i < k and c[k] for the centre.
+template <typename C, int NQ>
+struct StiffTab {
+  static constexpr int H = NQ / 2, HE = (NQ + 1) / 2, RE = HE - 1, RO = H;
+  C e[RE > 1 ? RE * (RE - 1) / 2 : 1];
+  C c[RE > 0 ? RE : 1];
+  C o[RO > 1 ? RO * (RO - 1) / 2 : 1];
+};
+
+// d L^T of one direction, its metric factor included: e[k (k+1)/2 + i] for the
+// parts i <= k, c[k] for the centre.
+template <typename C, int NQ>
+struct StiffBack {
+  using T = StiffTab<C, NQ>;
+  C e[T::RE > 0 ? T::RE * (T::RE + 1) / 2 : 1];
+  C c[T::RE > 0 ? T::RE : 1];
+  C o[T::RO * (T::RO + 1) / 2];
+};
+
 // Tables of the box kernel for C coefficients.  N: nodes to points, Nt its
-// transpose; K maps
-// (even, odd) parts to (even, odd) parts.
+// transpose; K maps (even, odd) parts to (even, odd) parts.
 template <typename C, int NP, int NQ>
 struct BoxTables {
   EOTab<C, NQ, NP> N;
   EOTab<C, NP, NQ> Nt;
-  EOTab<C, NQ, NQ> Kx, Ky, Kz;
+  StiffTab<C, NQ> K;
+  StiffBack<C, NQ> kx, ky, kz;
 };
+
+// One half of s (+)= L^T d L t over R rows; CENTRE: the even half, with its
+// centre t[R] and s[R].  (ADD: see eo_row.)
+template <typename A, int R, bool CENTRE, bool ADD, typename TC>
+__device__ __forceinline__ void stiff_half(const TC* l, const TC* lc, const TC* b, const TC* bc,
+                                           const typename A::V* t, typename A::V* s) {
+  if constexpr (R > 0) {
+    typename A::V y[R];
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+      typename A::Acc a = A::init(t[k]);
+#pragma unroll
+      for (int i = 0; i < k; ++i) A::fma(a, l[k * (k - 1) / 2 + i], t[i]);
+      if constexpr (CENTRE) A::fma(a, lc[k], t[R]);
+      y[k] = CENTRE || k > 0 ? A::value(a) : t[k];
+    }
+    constexpr bool kFromSum = ADD && !A::kSumApart;
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      typename A::Acc a = kFromSum ? A::init(s[i]) : A::first(b[i * (i + 1) / 2 + i], y[i]);
+#pragma unroll
+      for (int k = kFromSum ? i : i + 1; k < R; ++k) A::fma(a, b[k * (k + 1) / 2 + i], y[k]);
+      s[i] = ADD && !kFromSum ? A::add(s[i], A::value(a)) : A::value(a);
+    }
+    if constexpr (CENTRE) eo_row<A, R, ADD>(bc, y, s[R]);
+  } else if constexpr (CENTRE && !ADD) {
+    s[0] = A::zero();
+  }
+}
+
+// s (+)= K t on (even, odd) parts, b of one direction.
+template <typename A, int NQ, bool ADD = false>
+__device__ __forceinline__ void stiff_parts(const StiffTab<typename A::C, NQ>& K,
+                                            const StiffBack<typename A::C, NQ>& b, const typename A::V* t,
+                                            typename A::V* s) {
+  using T = StiffTab<typename A::C, NQ>;
+  stiff_half<A, T::RE, true, ADD>(K.e, K.c, b.e, b.c, t, s);
+  stiff_half<A, T::RO, false, ADD>(K.o, K.o, b.o, b.o, t + T::HE, s + T::HE);
+}
 
 // One cell e and B groups of W vectors: thread (v, ty) of B x nty threads
 // works on group vb B + v.  Switches: SC the scaled
@@ -112,7 +184,7 @@ __device__ __forceinline__ void cell_body_box(const BoxTables<typename Arith<V>:
     for (int i = 0; i < NP; ++i) u[i] = T[i * PP + at];
     eo_split<A, NP>(u, ue, uo);
     eo_parts<A, NQ, NP>(tab.N, ue, uo, t);
-    eo_parts<A, NQ, NQ>(tab.Kz, t, t + HQ, s);
+    stiff_parts<A, NQ>(tab.K, tab.kz, t, s);
     eo_join<A, NQ>(t);
     eo_join<A, NQ>(s);
 #pragma unroll
@@ -131,7 +203,7 @@ __device__ __forceinline__ void cell_body_box(const BoxTables<typename Arith<V>:
       t[q] = T[q * RP + at];
       s[q] = S[q * RP + at];
     }
-    eo_parts<A, NQ, NQ, true>(tab.Ky, t, t + HQ, s);
+    stiff_parts<A, NQ, true>(tab.K, tab.ky, t, s);
     eo_join<A, NQ>(t);
     eo_join<A, NQ>(s);
 #pragma unroll
@@ -154,7 +226,7 @@ __device__ __forceinline__ void cell_body_box(const BoxTables<typename Arith<V>:
       t[q] = line[q];
       s[q] = S[l * RP + q];
     }
-    eo_parts<A, NQ, NQ, true>(tab.Kx, t, t + HQ, s);
+    stiff_parts<A, NQ, true>(tab.K, tab.kx, t, s);
     eo_join<A, NQ>(t);
     // the mirrored sums and differences N^T needs; those of s's values are
     // twice its parts (once at the middle point)
@@ -230,19 +302,31 @@ __global__ void __launch_bounds__(256) cell_apply_box_local_kernel(
                                                reinterpret_cast<V*>(smem_raw), Scale<typename Arith<V>::D>{});
 }
 
-// Host: (even, odd)-part table of f K (see fe_ctx::Ks).
+// Host: L, and f d L^T (see fe_ctx::KLe; a middle point stands once where a
+// pair stands twice).
 template <typename C, int NQ>
-void make_stiffness(EOTab<C, NQ, NQ>& t, const fe_ctx* c, double f) {
-  constexpr int H = NQ / 2, HE = (NQ + 1) / 2;
-  for (int o = 0; o < HE; ++o) {
-    for (int i = 0; i < HE; ++i) t.E[o][i] = (C)(f * c->Ks[o * HE + i]);
-    for (int i = 0; i < H; ++i) t.O[o][i] = (C)(f * c->Kd[o * HE + i]);
-  }
+void make_stiffness(StiffTab<C, NQ>& t, const fe_ctx* c) {
+  for (size_t i = 0; i < c->KLe.size(); ++i) t.e[i] = (C)c->KLe[i];
+  for (size_t i = 0; i < c->KLc.size(); ++i) t.c[i] = (C)c->KLc[i];
+  for (size_t i = 0; i < c->KLo.size(); ++i) t.o[i] = (C)c->KLo[i];
+}
+
+template <typename C, int NQ>
+void make_stiffness_back(StiffBack<C, NQ>& t, const fe_ctx* c, double f) {
+  auto half = [f](C* b, const std::vector<double>& L, const std::vector<double>& d) {
+    const int R = (int)d.size();
+    for (int k = 0; k < R; ++k)
+      for (int i = 0; i <= k; ++i)
+        b[k * (k + 1) / 2 + i] = (C)(f * d[k] * (i == k ? 1.0 : L[k * (k - 1) / 2 + i]));
+  };
+  half(t.e, c->KLe, c->KDe);
+  half(t.o, c->KLo, c->KDo);
+  for (size_t k = 0; k < c->KDe.size(); ++k) t.c[k] = (C)((NQ & 1 ? 2.0 : 1.0) * f * c->KDe[k] * c->KLc[k]);
 }
 
 template <typename C, int NP, int NQ>
 BoxTables<C, NP, NQ> make_boxtables(const fe_ctx* c) {
-  BoxTables<C, NP, NQ> t;
+  BoxTables<C, NP, NQ> t{};
   double Nt[NP * NQ];
   for (int q = 0; q < NQ; ++q)
     for (int i = 0; i < NP; ++i) Nt[i * NQ + q] = c->Nf[q * NP + i];
@@ -250,9 +334,10 @@ BoxTables<C, NP, NQ> make_boxtables(const fe_ctx* c) {
   make_eotab(t.Nt, Nt);
   // g_dd = mu det J (2 / h_d)^2
   const double* h = c->box_h;
-  make_stiffness(t.Kx, c, (h[2] / h[0]) * (h[2] / h[0]));
-  make_stiffness(t.Ky, c, (h[2] / h[1]) * (h[2] / h[1]));
-  make_stiffness(t.Kz, c, 1.0);
+  make_stiffness(t.K, c);
+  make_stiffness_back(t.kx, c, (h[2] / h[0]) * (h[2] / h[0]));
+  make_stiffness_back(t.ky, c, (h[2] / h[1]) * (h[2] / h[1]));
+  make_stiffness_back(t.kz, c, 1.0);
   return t;
 }
 

@@ -63,7 +63,8 @@ __device__ __forceinline__ void eo_join(typename A::V* x) {
 // products are added to what out holds.  Double-float and FP32 sum the products
 // first and add the sum: what out holds is larger than one direction's share,
 // and every term added to it would be rounded at its scale (the double-float
-// error of a p = 6 product is 1.2e-14 this way, 1.4e-14 the other).  FP64
+// error of a p = 6 product was 1.2e-14 this way, 1.4e-14 the other, with the
+// stiffness as one matrix).  FP64
 // starts its sum from it: one operation less on the pipe that bounds it.
 template <typename A, int NI, typename TC, typename TV>
 __device__ __forceinline__ typename A::V eo_dot(const TC* c, const TV* x) {

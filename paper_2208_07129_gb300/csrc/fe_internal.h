@@ -115,9 +115,12 @@ struct fe_ctx {
   // host FP64 data
   std::vector<double> gll, wgll, qx, qw, N1, D1;   // N1[q*np+i], D1[q*nq+k] (unfolded)
   std::vector<double> Nf, Df;                // folded
-  // stiffness at the points, K = Df^T Df: K[i][j] + K[i][nq-1-j] and the
-  // difference, i < (nq+1)/2, j < nq/2, then the middle column (box kernel)
-  std::vector<double> Ks, Kd;
+  // Stiffness at the points, K = Df^T Df, by its halves on (even, odd) parts,
+  // each factored as L^T d L with unit lower triangular L (box kernel).  Even:
+  // row p < RE = (nq+1)/2 - 1 of L has KLe[p (p-1)/2 + i] for the parts i < p and
+  // KLc[p] for the centre (the middle pair, or point), which has no row of its
+  // own: K annihilates sqrt(w), the constant.  Odd: rows p < nq/2 of KLo.
+  std::vector<double> KLe, KLc, KDe, KLo, KDo;
   std::vector<double> vertices;              // copy of the vertex array (general)
   double box_lo[3] = {0, 0, 0}, box_h[3] = {1, 1, 1};  // uniform box: corner and cell size
   std::vector<double> detJ;                  // per point (E*nq3)

@@ -192,24 +192,49 @@ void build_tables(fe_ctx* c) {
   build_stiffness(c);
 }
 
-// Ks, Kd: extended precision, so that forming the matrix adds one rounding to
-// those of the folded table.
+// The factors of the stiffness at the points (see fe_ctx::KLe).  Everything is
+// formed in extended precision, so that a factor carries little more than one
+// rounding beside those of the folded table.
 static void build_stiffness(fe_ctx* c) {
-  const int nq = c->nq, HE = (nq + 1) / 2, H = nq / 2;
+  const int nq = c->nq, HE = (nq + 1) / 2, H = nq / 2, RE = HE - 1;
   auto k = [&](int a, int b) {
     long double s = 0.0L;
     for (int q = 0; q < nq; ++q) s += (long double)c->Df[q * nq + a] * c->Df[q * nq + b];
     return s;
   };
-  c->Ks.assign((size_t)HE * HE, 0.0);
-  c->Kd.assign((size_t)HE * HE, 0.0);
-  for (int o = 0; o < HE; ++o) {
-    for (int i = 0; i < H; ++i) {
-      c->Ks[o * HE + i] = (double)(k(o, i) + k(o, nq - 1 - i));
-      c->Kd[o * HE + i] = (double)(k(o, i) - k(o, nq - 1 - i));
+  // B = L^T d L for the first `rank` of n indices, taken from the last of them
+  // down; column n - 1 holds the centre when rank < n
+  auto factor = [](std::vector<long double>& B, int n, int rank, std::vector<double>& L, std::vector<double>& centre,
+                   std::vector<double>& d) {
+    L.assign((size_t)rank * (rank > 0 ? rank - 1 : 0) / 2, 0.0);
+    centre.assign(rank < n ? rank : 0, 0.0);
+    d.assign(rank, 0.0);
+    for (int p = rank - 1; p >= 0; --p) {
+      const long double dp = B[p * n + p];
+      d[p] = (double)dp;
+      for (int i = 0; i < n; ++i) {
+        if (i == p || (i > p && i < rank)) continue;
+        const long double l = B[p * n + i] / dp;
+        (i < p ? L[(size_t)p * (p - 1) / 2 + i] : centre[p]) = (double)l;
+        for (int j = 0; j < n; ++j)
+          if (j != p && !(j > p && j < rank)) B[i * n + j] -= l * B[p * n + j];
+      }
     }
-    if (HE > H) c->Ks[o * HE + H] = (double)k(o, H);
-  }
+  };
+  // even half: pairs i, nq-1-i weigh twice a middle point in the energy; half
+  // of it is kept, so that d belongs to the pairs' parts
+  std::vector<long double> B((size_t)HE * HE);
+  for (int o = 0; o < HE; ++o)
+    for (int i = 0; i < HE; ++i) {
+      const bool mo = o >= H, mi = i >= H;   // the middle point
+      B[o * HE + i] = mo && mi ? 0.5L * k(o, i) : mi ? k(o, i) : mo ? k(o, i) : k(o, i) + k(o, nq - 1 - i);
+    }
+  factor(B, HE, RE, c->KLe, c->KLc, c->KDe);
+  B.assign((size_t)H * H, 0.0L);
+  for (int o = 0; o < H; ++o)
+    for (int i = 0; i < H; ++i) B[o * H + i] = k(o, i) - k(o, nq - 1 - i);
+  std::vector<double> none;
+  factor(B, H, H, c->KLo, none, c->KDo);
 }
 
 double lagrange_1d(const double* xs, int n, int k, double t) { return lagrange_value(xs, n, k, t); }
