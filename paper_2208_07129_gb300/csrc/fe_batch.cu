@@ -18,6 +18,7 @@
 // item) that keeps the queue several items deep per SM.
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <map>
 #include <vector>
@@ -39,7 +40,7 @@ template <typename T>
 struct BatchProblemDev {
   MeshDev m;
   Geom<typename Arith<T>::G> geo;
-  int n_vec, vb, nty, kind, n_vb;                      // vb: vectors per item
+  int n_vec, vb, kind, n_vb;                           // vb: vectors per item
   const int* cells;                                    // colour-sorted cell ids
   typename Arith<T>::C tab[kTabImage];                                    // BoxTables<T, NP, NQ> image
 };
@@ -54,13 +55,15 @@ constexpr int kind_of(int p) { return p - 3; }
 template <typename T, int NP, int NQ>
 __device__ __forceinline__ void run_item(const BatchProblemDev<T>& P, const WorkItem& w,
                                          const typename Arith<T>::D* X, typename Arith<T>::D* Y, T* smem,
-                                         const BoxTables<typename Arith<T>::C, NP, NQ>& tab) {
+                                         const BoxTables<typename Arith<T>::C, NP, NQ>& tab,
+                                         const StiffBack<typename Arith<T>::C, NQ>& kx,
+                                         const StiffBack<typename Arith<T>::C, NQ>& ky) {
   const int tid = threadIdx.x, lanes = P.vb / Arith<T>::W;
   const int v = tid % lanes, ty = tid / lanes, nty = kBatchThreads / lanes;
   const bool vec = vec_ok<T>(X, Y, P.n_vec);
   for (int c = 0; c < w.cell_count; ++c) {
     const int e = P.cells[w.cell_begin + c];
-    cell_body_box<T, NP, NQ>(tab, P.m, P.geo, e, w.vb, lanes, v, ty, nty, P.n_vec, vec, X, Y, smem,
+    cell_body_box<T, NP, NQ>(tab, kx, ky, P.m, P.geo, e, w.vb, lanes, v, ty, nty, P.n_vec, vec, X, Y, smem,
                              Scale<typename Arith<T>::D>{});
     __syncthreads();
   }
@@ -72,20 +75,29 @@ __device__ __forceinline__ unsigned long long batch_clock_ns() {
   return t;
 }
 
-// One persistent kernel per group of problems of one degree and one aspect of
-// their cells (which share the 1D tables), with its own queue: each
-// instantiation gets the registers its cell body needs instead of those of
-// the largest degree in the batch, and the group's tables travel as a kernel parameter, so the
-// contractions read their coefficients from the constant bank as in the
-// per-colour kernels.
-template <typename T, int NP, int NQ>
+// One persistent kernel per group of problems, those of one degree, with its
+// own queue: each instantiation gets the registers its cell body needs instead
+// of those of the largest degree in the batch, and the group's tables travel as
+// a kernel parameter, so the contractions read their coefficients from the
+// constant bank as in the per-colour kernels.  Of the tables only d L^T along x
+// and y depend on the aspect of a mesh's cells; in a group whose problems
+// differ in it (MIXED) each item brings its problem's two in shared memory.
+// 24 problems of 8^3 cells, p = 4, 32 vectors with one aspect and with 24:
+// double-float 1.56 and 1.63 ms, FP32 0.46 and 0.51; p = 3, 64 vectors: 1.47 and
+// 1.70, 0.46 and 0.64, so the constant bank stays where it serves.  (A kernel
+// per aspect left each colour's tail idle: 8..10 x 8 x 8 cells, p = 4, 24 times
+// three aspects 5.66 and 1.56 ms, this way 1.82 and 0.57.)
+template <typename T, int NP, int NQ, bool MIXED>
 __global__ void __launch_bounds__(kBatchThreads) batch_kernel(const BoxTables<typename Arith<T>::C, NP, NQ> tab,
                                                              const BatchProblemDev<T>* __restrict__ probs,
                                                              const void* const* __restrict__ ptrs,
                                                              const WorkItem* __restrict__ items, int n_items,
                                                              int* next, int* done, const int* __restrict__ need,
                                                              int* status, const long long* __restrict__ wait_ns) {
+  using C = typename Arith<T>::C;
+  using Back = StiffBack<C, NQ>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ __align__(16) C s_back[MIXED ? 2 * (sizeof(Back) / sizeof(C)) : 1];   // kx, ky
   __shared__ int s_item;
   T* smem = reinterpret_cast<T*>(smem_raw);
   for (;;) {
@@ -108,11 +120,17 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(const BoxTables<ty
       }
       __threadfence();
     }
+    if constexpr (MIXED) {
+      using Tab = BoxTables<C, NP, NQ>;
+      constexpr int first = offsetof(Tab, kx) / sizeof(C);
+      for (int k = threadIdx.x; k < (int)(2 * sizeof(Back) / sizeof(C)); k += blockDim.x) s_back[k] = P.tab[first + k];
+    }
     __syncthreads();
     using D = typename Arith<T>::D;
     const D* X = static_cast<const D*>(ptrs[2 * w.problem]);
     D* Y = static_cast<D*>(const_cast<void*>(ptrs[2 * w.problem + 1]));
-    run_item<T, NP, NQ>(P, w, X, Y, smem, tab);
+    const Back* back = reinterpret_cast<const Back*>(s_back);
+    run_item<T, NP, NQ>(P, w, X, Y, smem, tab, MIXED ? back[0] : tab.kx, MIXED ? back[1] : tab.ky);
     if (threadIdx.x == 0) {
       __threadfence();
       atomicAdd(&done[w.problem * kMaxColors + w.color], 1);
@@ -123,8 +141,8 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(const BoxTables<ty
 
 
 // FP64: one persistent kernel for every degree, the tables of each item's
-// problem staged in shared memory.  Measured faster than the per-degree
-// kernels for FP64 (950 against 1030 ms on the 24-problem batch): the FP64
+// problem staged in shared memory.  Measured faster than a kernel per group
+// for FP64 (18.0 against 23.0 ms on six problems of 5 to 20 cells): the FP64
 // pipe bounds both, and one kernel keeps every degree's work in flight
 // together.  Its register allocation is the largest degree's, which costs the
 // double-float and FP32 cell bodies much more than it costs FP64.
@@ -163,8 +181,12 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel_all(const BatchPro
     using D = typename Arith<T>::D;
     const D* X = static_cast<const D*>(ptrs[2 * w.problem]);
     D* Y = static_cast<D*>(const_cast<void*>(ptrs[2 * w.problem + 1]));
-#define FE_ITEM(K, NP, NQ) \
-  case K: run_item<T, NP, NQ>(P, w, X, Y, smem, *reinterpret_cast<const BoxTables<typename Arith<T>::C, NP, NQ>*>(stab)); break;
+#define FE_ITEM(K, NP, NQ)                                                                                  \
+  case K: {                                                                                                 \
+    const auto& tab = *reinterpret_cast<const BoxTables<typename Arith<T>::C, NP, NQ>*>(stab);               \
+    run_item<T, NP, NQ>(P, w, X, Y, smem, tab, tab.kx, tab.ky);                                              \
+    break;                                                                                                  \
+  }
     switch (P.kind) {
       FE_ITEM(0, 4, 5) FE_ITEM(1, 5, 6) FE_ITEM(2, 6, 7) FE_ITEM(3, 7, 8) FE_ITEM(4, 8, 9) FE_ITEM(5, 9, 10)
       default: break;
@@ -191,9 +213,10 @@ struct fe_batch {
   WorkItem* d_items = nullptr;
   int n_items = 0, n_phases = 0;
   // groups of problems that share one kernel and its queue: one for every
-  // problem in FP64, else one per degree and cell aspect
+  // problem in FP64, else one per degree
   std::vector<int> group_of;           // group of each problem
   std::vector<int> group_first;        // a problem of each group (its tables are the group's)
+  std::vector<char> group_mixed;       // its problems differ in the aspect of their cells
   std::vector<int> item_begin;         // items of group g: [item_begin[g], item_begin[g + 1])
   int *d_next = nullptr, *d_done = nullptr, *d_need = nullptr, *d_status = nullptr;
   std::vector<int> need;               // host copy of the completion counts items wait for
@@ -303,8 +326,13 @@ int autotune(const fe_ctx* c, int n_vec_full, fe_mode mode, float* spent_ms) {
 // attribute and its grid = occupancy x SMs (at most one CTA per work item);
 // then its launch, recorded into the graph.
 template <typename T, int NP, int NQ>
+auto group_kernel(const fe_batch* b, int g) {
+  return b->group_mixed[g] ? batch_kernel<T, NP, NQ, true> : batch_kernel<T, NP, NQ, false>;
+}
+
+template <typename T, int NP, int NQ>
 cudaError_t prepare_group(fe_batch* b, int g, int n_g, size_t smem) {
-  auto kern = batch_kernel<T, NP, NQ>;
+  auto kern = group_kernel<T, NP, NQ>(b, g);
   cudaError_t e = ensure_dyn_smem(reinterpret_cast<const void*>(kern), smem);
   int per_sm = 0, sms = 0, dev = 0;
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kBatchThreads, smem);
@@ -318,7 +346,7 @@ cudaError_t prepare_group(fe_batch* b, int g, int n_g, size_t smem) {
 
 template <typename T, int NP, int NQ>
 cudaError_t launch_group(fe_batch* b, int g, int n_g, size_t smem) {
-  auto kern = batch_kernel<T, NP, NQ>;
+  auto kern = group_kernel<T, NP, NQ>(b, g);
   using C = typename Arith<T>::C;
   const BoxTables<C, NP, NQ> tab = make_boxtables<C, NP, NQ>(b->ctxs[b->group_first[g]]);
   kern<<<b->group_grid[g], kBatchThreads, smem, b->side[g]>>>(
@@ -342,10 +370,10 @@ cudaError_t for_group(fe_batch* b, int g, size_t smem, bool launch) {
   }
 }
 
-// Whether two problems share their 1D tables: the degree (and so n_q) and the
-// cells' aspect (the stiffness tables carry its ratios).
-bool same_tables(const fe_ctx* a, const fe_ctx* b) {
-  return a->p == b->p && a->box_h[2] / a->box_h[0] == b->box_h[2] / b->box_h[0] &&
+// Whether two problems of a degree share all their 1D tables: the cells' aspect
+// (the stiffness tables of x and y carry its ratios).
+bool same_aspect(const fe_ctx* a, const fe_ctx* b) {
+  return a->box_h[2] / a->box_h[0] == b->box_h[2] / b->box_h[0] &&
          a->box_h[2] / a->box_h[1] == b->box_h[2] / b->box_h[1];
 }
 
@@ -379,7 +407,6 @@ fe_status build_batch(fe_batch* b, int autotune_on) {
       tuned[key] = vb;
     }
     P.vb = vb;
-    P.nty = kBatchThreads / vb;
     P.n_vb = (P.n_vec + vb - 1) / vb;
     b->vb[i] = vb;
     std::memset(P.tab, 0, sizeof(P.tab));
@@ -394,16 +421,20 @@ fe_status build_batch(fe_batch* b, int autotune_on) {
     }
     smem = std::max(smem, tile_smem<T>(c->nq, vb));
   }
-  // groups: every problem (FP64, merged kernel), or the problems that share
-  // their tables (one kernel and one queue each)
+  // groups: every problem (FP64, merged kernel), or the problems of one degree
+  // (one kernel and one queue each)
   constexpr bool merged = std::is_same<T, double>::value;
   b->group_of.assign(n, 0);
   for (int i = 0; i < n; ++i) {
     int g = 0;
     const int ng = (int)b->group_first.size();
-    while (g < ng && !merged && !same_tables(b->ctxs[b->group_first[g]], b->ctxs[i])) ++g;
-    if (g == ng) b->group_first.push_back(i);
+    while (g < ng && !merged && b->ctxs[b->group_first[g]]->p != b->ctxs[i]->p) ++g;
+    if (g == ng) {
+      b->group_first.push_back(i);
+      b->group_mixed.push_back(0);
+    }
     b->group_of[i] = g;
+    if (!same_aspect(b->ctxs[b->group_first[g]], b->ctxs[i])) b->group_mixed[g] = 1;
   }
   const int groups = (int)b->group_first.size();
   b->group_grid.assign(groups, 0);

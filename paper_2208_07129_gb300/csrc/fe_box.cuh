@@ -125,12 +125,14 @@ __device__ __forceinline__ void stiff_parts(const StiffTab<typename A::C, NQ>& K
 }
 
 // One cell e and B groups of W vectors: thread (v, ty) of B x nty threads
-// works on group vb B + v.  Switches: SC the scaled
+// works on group vb B + v.  kx, ky: tab's, or those of another mesh of the degree.  Switches: SC the scaled
 // product, MAP the explicit map of refined meshes, LOCAL the per-cell scratch.
 // vec: X, Y and n_vec are multiples of W values (set by the launch), so a
 // group moves in one access.
 template <typename V, int NP, int NQ, bool SC = false, bool MAP = false, bool LOCAL = false>
-__device__ __forceinline__ void cell_body_box(const BoxTables<typename Arith<V>::C, NP, NQ>& tab, const MeshDev& m,
+__device__ __forceinline__ void cell_body_box(const BoxTables<typename Arith<V>::C, NP, NQ>& tab,
+                                              const StiffBack<typename Arith<V>::C, NQ>& kx,
+                                              const StiffBack<typename Arith<V>::C, NQ>& ky, const MeshDev& m,
                                               const Geom<typename Arith<V>::G>& geo, int e, int vb, int B, int v,
                                               int ty, int nty, int n_vec, bool vec,
                                               const typename Arith<V>::D* __restrict__ X,
@@ -203,7 +205,7 @@ __device__ __forceinline__ void cell_body_box(const BoxTables<typename Arith<V>:
       t[q] = T[q * RP + at];
       s[q] = S[q * RP + at];
     }
-    stiff_parts<A, NQ, true>(tab.K, tab.ky, t, s);
+    stiff_parts<A, NQ, true>(tab.K, ky, t, s);
     eo_join<A, NQ>(t);
     eo_join<A, NQ>(s);
 #pragma unroll
@@ -226,7 +228,7 @@ __device__ __forceinline__ void cell_body_box(const BoxTables<typename Arith<V>:
       t[q] = line[q];
       s[q] = S[l * RP + q];
     }
-    stiff_parts<A, NQ, true>(tab.K, tab.kx, t, s);
+    stiff_parts<A, NQ, true>(tab.K, kx, t, s);
     eo_join<A, NQ>(t);
     // the mirrored sums and differences N^T needs; those of s's values are
     // twice its parts (once at the middle point)
@@ -284,7 +286,7 @@ __global__ void __launch_bounds__(256) cell_apply_box_kernel(
     typename Arith<V>::D* __restrict__ Y, const Scale<typename Arith<V>::D> sc, const int* __restrict__ map) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   let_next_launch_start();
-  cell_body_box<V, NP, NQ, SC, MAP>(tab, m, geo, cells[blockIdx.x / n_vb], blockIdx.x % n_vb, blockDim.x,
+  cell_body_box<V, NP, NQ, SC, MAP>(tab, tab.kx, tab.ky, m, geo, cells[blockIdx.x / n_vb], blockIdx.x % n_vb, blockDim.x,
                                     threadIdx.x, threadIdx.y, blockDim.y, n_vec, vec, X, Y,
                                     reinterpret_cast<V*>(smem_raw),
                                     sc, map);
@@ -297,7 +299,7 @@ __global__ void __launch_bounds__(256) cell_apply_box_local_kernel(
     int n_vec, int n_vb, bool vec, const typename Arith<V>::D* __restrict__ X, typename Arith<V>::D* __restrict__ Wk) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   let_next_launch_start();
-  cell_body_box<V, NP, NQ, false, false, true>(tab, m, geo, blockIdx.x / n_vb, blockIdx.x % n_vb, blockDim.x,
+  cell_body_box<V, NP, NQ, false, false, true>(tab, tab.kx, tab.ky, m, geo, blockIdx.x / n_vb, blockIdx.x % n_vb, blockDim.x,
                                                threadIdx.x, threadIdx.y, blockDim.y, n_vec, vec, X, Wk,
                                                reinterpret_cast<V*>(smem_raw), Scale<typename Arith<V>::D>{});
 }
