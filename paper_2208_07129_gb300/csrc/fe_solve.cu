@@ -82,8 +82,8 @@ cudaError_t col_dot(const T* a, const T* b, size_t n, int nv, const SolveWs& w, 
 
 constexpr int kWideBlocks = 152 * 8;
 // The reductions take 2 CTAs per SM with four rows in flight per thread: the sum
-// over threads and CTAs is the slow part (FP64 runs at 1/64 of the FP32 rate): with
-// 8 CTAs per SM joined in FP64 a 100 MB dot product took 68 us.
+// over threads and CTAs is the slow part (FP64 runs at 1/64 of the FP32 rate), and
+// 8 CTAs per SM have four times as much of it: a 100 MB dot product took 68 us.
 constexpr int kWideRedBlocks = 152 * 2;
 constexpr int kWideRows = 4;
 
@@ -132,25 +132,22 @@ inline bool wide_ok(int nv, const void* const* ptrs, int n_ptrs) {
 // Per-thread column sums of products.  FP64 blocks accumulate in FP64.  FP32
 // blocks accumulate in FP32 with Kahan's compensation (the running error is
 // fed back into the next term, so the sum is accurate to a few FP32 ulps
-// whatever its length) and are joined over the CTA in double-float, converted to
-// FP64 once per CTA: GB300 runs FP64 at 1/64 of the FP32 rate, and two conversions
-// plus an FP64 multiply-add per element would bound these streaming kernels.
+// whatever its length: 3.1e-10 of the terms' sum for 5 rows a thread, 2.9e-10 for
+// 20); the threads' sums are joined in FP64.  GB300 runs FP64 at 1/64 of the
+// FP32 rate, and two conversions plus an FP64 multiply-add per element would
+// bound these streaming kernels; per thread they are 0.5 % of the mixed solve
+// below (148.2 ms joined in double-float, 149.0 in FP64), which is paid for the
+// five bits.
 template <typename T>
 struct ColAcc;
 template <>
 struct ColAcc<double> {
-  using Part = double;   // a thread's sum, summed over the CTA
-  static __device__ Part join(Part a, Part b) { return a + b; }
-  static __device__ double out(Part a) { return a; }
   double s = 0.0;
   __device__ void add(double a, double b) { s = fma(a, b, s); }
-  __device__ Part value() const { return s; }
+  __device__ double value() const { return s; }
 };
 template <>
 struct ColAcc<float> {
-  using Part = ff;       // s - c exactly; double-float sums keep 48 bits
-  static __device__ Part join(Part a, Part b) { return ff_add(a, b); }
-  static __device__ double out(Part a) { return ff_to_double(a); }
   float s = 0.f, c = 0.f;
   __device__ void add(float a, float b) {
     const float y = __fsub_rn(__fmul_rn(a, b), c);
@@ -158,7 +155,7 @@ struct ColAcc<float> {
     c = __fsub_rn(__fsub_rn(t, s), y);
     s = t;
   }
-  __device__ Part value() const { return renorm(s, -c); }
+  __device__ double value() const { return (double)s - (double)c; }
 };
 
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
@@ -192,8 +189,7 @@ template <typename T>
 __device__ __forceinline__ void wide_finish(const ColAcc<T> (&acc)[Wide<T>::N], bool col_ok, int cg, int nv,
                                             double* __restrict__ partial, const ColScalar& o) {
   constexpr int N = Wide<T>::N;
-  using Part = typename ColAcc<T>::Part;
-  __shared__ Part red[256][N];
+  __shared__ double red[256][N];
   __shared__ bool last;
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
 #pragma unroll
@@ -202,12 +198,12 @@ __device__ __forceinline__ void wide_finish(const ColAcc<T> (&acc)[Wide<T>::N], 
     __syncthreads();
     if ((int)threadIdx.y < h) {
 #pragma unroll
-      for (int k = 0; k < N; ++k) red[tid][k] = ColAcc<T>::join(red[tid][k], red[tid + h * blockDim.x][k]);
+      for (int k = 0; k < N; ++k) red[tid][k] += red[tid + h * blockDim.x][k];
     }
   }
   if (threadIdx.y == 0 && col_ok) {
 #pragma unroll
-    for (int k = 0; k < N; ++k) partial[(size_t)blockIdx.x * nv + cg * N + k] = ColAcc<T>::out(red[tid][k]);
+    for (int k = 0; k < N; ++k) partial[(size_t)blockIdx.x * nv + cg * N + k] = red[tid][k];
   }
   __threadfence();
   __syncthreads();
