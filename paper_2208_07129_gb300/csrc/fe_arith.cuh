@@ -95,7 +95,8 @@ struct Arith<double> {
 
 // Two FP32 vectors per value, on the packed FP32 instructions of sm_100: one
 // issue slot for two operations, and half the shared-memory and global accesses.
-// A lane's results are those of the scalar operations.  FP32 was bound by
+// A lane's results are those of the scalar operations (a product that is -0
+// comes out as +0).  FP32 was bound by
 // issue: 16^3 p = 6, n_q = 8, 64 vectors 0.728 -> 0.464 ms.  Four vectors per
 // value take 118 registers and gained only for n_q <= 6 (0.36 -> 0.32 ms at
 // 20^3 p = 4, but 0.46 -> 0.49 ms at p = 6).  Double-float stays on one vector:

@@ -88,16 +88,16 @@ __device__ __forceinline__ void eo_row(const TC* c, const typename A::V* x, type
   }
 }
 
-template <typename A, int NO, int NI, bool ADD = false>
+template <typename A, int NO, int NI>
 __device__ __forceinline__ void eo_parts(const EOTab<typename A::C, NO, NI>& t, const typename A::V* e,
                                          const typename A::V* o, typename A::V* out) {
   constexpr int HI = NI / 2, HE = (NI + 1) / 2, HO = (NO + 1) / 2;
 #pragma unroll
-  for (int k = 0; k < HO; ++k) eo_row<A, HE, ADD>(t.E[k], e, out[k]);
+  for (int k = 0; k < HO; ++k) eo_row<A, HE, false>(t.E[k], e, out[k]);
 #pragma unroll
   for (int k = 0; k < NO / 2; ++k) {
-    if constexpr (HI > 0) eo_row<A, HI, ADD>(t.O[k], o, out[HO + k]);
-    else if (!ADD) out[HO + k] = A::zero();
+    if constexpr (HI > 0) eo_row<A, HI, false>(t.O[k], o, out[HO + k]);
+    else out[HO + k] = A::zero();
   }
 }
 

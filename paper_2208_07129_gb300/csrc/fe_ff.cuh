@@ -50,14 +50,6 @@ __device__ __forceinline__ ff ff_add(ff a, ff b) {
 
 __device__ __forceinline__ ff ff_sub(ff a, ff b) { return ff_add(a, ff(-b.hi, -b.lo)); }
 
-__device__ __forceinline__ ff ff_mul(ff a, ff b) {
-  const float p = __fmul_rn(a.hi, b.hi);
-  float e = __fmaf_rn(a.hi, b.hi, -p);
-  e = __fmaf_rn(a.hi, b.lo, e);
-  e = __fmaf_rn(a.lo, b.hi, e);
-  return renorm(p, e);
-}
-
 // Compensated dot-product accumulator: value s + c.
 struct ffacc {
   float s, c;

@@ -91,15 +91,6 @@ struct SolveWs {
 
 struct LearnedPrecond;
 
-struct KernelLaunch {
-  const int* cells;   // cell ids of this colour (device)
-  int n_cells;
-  int n_vec;
-  int vb;             // vectors per CTA
-  int nty;            // lines in flight per CTA (blockDim.y)
-  cudaStream_t stream;
-};
-
 }  // namespace fe
 
 // Floats per cell of fe_ctx::d_ptCtc: 8 planes of 72 (64 values, 8 of padding).
@@ -174,7 +165,7 @@ struct fe_ctx {
   void* blas = nullptr;
   void* solver = nullptr;
   // launch shape per mode (vectors per CTA, lines per CTA)
-  int vb64 = 8, nty64 = 16, vb32 = 8, nty32 = 32, vbdf = 8, ntydf = 32;
+  int vb64 = 8, nty64 = 16, vb32 = 8, nty32 = 32, vbdf = 0, ntydf = 0;
   // the box kernel has its own defaults (Arith::box_tile) until fe_set_tile sets a tile
   bool set64 = false, set32 = false, setdf = false;
   fe::LineTile tile64() const { return set64 ? fe::LineTile{vb64, nty64} : fe::LineTile{0, 0}; }

@@ -98,7 +98,6 @@ extern "C" fe_status fe_setup_refined(const fe_refined_desc* md, int p, const fe
   c->periodic = 0;
   c->p = p; c->np = p + 1; c->nq = quad->n_q; c->quad_kind = quad->kind; c->mu = mu;
   c->general = 0;
-  if (quad->n_q >= 9) { c->vb64 = 4; c->nty64 = 32; c->vb32 = 4; c->nty32 = 64; c->vbdf = 4; c->ntydf = 64; }
   c->fp32_variant = 3;
   build_tables(c);
   const int np = c->np, nq = c->nq, NP3 = np * np * np;

@@ -348,7 +348,7 @@ extern "C" fe_status fe_setup(const fe_mesh_desc* mesh, int p, const fe_quad_des
   // vectors x 16 lines up to n_q = 8, 4 x 32 above; FP32 8 x 32 and 4 x 64.  The
   // default kernels have their own (Arith::box_tile, Arith::general_tile).
   c->fp32_variant = 3;
-  if (quad->n_q >= 9) { c->vb64 = 4; c->nty64 = 32; c->vb32 = 4; c->nty32 = 64; c->vbdf = 4; c->ntydf = 64; }
+  if (quad->n_q >= 9) { c->vb64 = 4; c->nty64 = 32; c->vb32 = 4; c->nty32 = 64; }
   const int np = c->np, nq = c->nq;
   const int add = c->periodic ? 0 : 1;
   c->mdev.nx = c->nx; c->mdev.ny = c->ny; c->mdev.nz = c->nz;
