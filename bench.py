@@ -190,9 +190,10 @@ FP64_KERNEL = "cell_apply_box_kernel<double,7,8>"
 def box_operations_per_cell_vec(np_: int, nq: int) -> int:
     """Operations (one FP64 pipe slot each: add, multiply or multiply-add) the
     box-cell kernel executes per cell and vector, pass by pass (fe_box.cuh):
-    even-odd contractions with N, the separable stiffness, and N^T."""
+    even-odd contractions with N, the separable stiffness in its factors, and
+    N^T."""
     hq, oq, hp, op = (nq + 1) // 2, nq // 2, (np_ + 1) // 2, np_ // 2
-    n, nt, k = hq * hp + oq * op, hp * hq + op * oq, hq * hq + oq * oq
+    n, nt, k = hq * hp + oq * op, hp * hq + op * oq, hq * hq - 1 + oq * oq   # k: L and d L^T of both halves
     point = 5 * oq + 2 * (nq & 1)
     return (np_ * np_ * (2 * op + n) + np_ * nq * (2 * op + n) + nq * nq * (2 * op + n + k + 4 * oq)
             + nq * nq * (k + 4 * oq) + nq * nq * (k + 2 * oq + point + nt + 2 * op)
@@ -485,7 +486,7 @@ def small_case_bench(fe, torch, steps: int = 50) -> dict:
             b.record()
             torch.cuda.synchronize()
             out[mode + "_us_per_apply"] = a.elapsed_time(b) / steps * 1e3
-        out["launches_per_apply"] = 8
+        out["launches_per_apply"] = 2   # every cell, then the colour-ordered gather
     finally:
         fe.fe_destroy(ctx)
     return out
