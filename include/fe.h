@@ -187,9 +187,10 @@ fe_mode fe_get_mode(const fe_ctx* ctx);
  * threads.  In FE_FP64, FE_DF64, FE_FP32 and FE_TF32X3 on structured meshes
  * they may also run on several streams and as replays of captured graphs at
  * the same time (small meshes keep a block of scratch for products outside
- * captures and one each for three pairs of capture and stream, given back with
- * the graph; a product that finds none free runs colour by colour, with the
- * same bits; a graph instantiated twice must not run beside itself).  In
+ * captures and one each for up to 16 pairs of capture and stream, allocated by
+ * the first product captured there and given back with the graph; a product
+ * that finds none free runs colour by colour, with the same bits; a graph
+ * instantiated twice must not run beside itself).  In
  * FE_TF32, FE_BF16 and FE_BF16S (task counters in the context) and on refined
  * meshes with hanging nodes (the block above) products on different streams
  * have to be ordered by the caller. */

@@ -17,19 +17,20 @@ struct SmallScratch::Captures {
 
 SmallScratch::~SmallScratch() {
   cudaFree(mem_);
+  for (char* m : captured_mem_) cudaFree(m);
   if (done_) cudaEventDestroy(done_);
 }
 
 cudaError_t SmallScratch::create(size_t block_bytes) {
   captures_ = std::make_shared<Captures>();
-  cudaError_t e = cudaMalloc(&mem_, (1 + kCaptures) * block_bytes);
+  cudaError_t e = cudaMalloc(&mem_, block_bytes);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&done_, cudaEventDisableTiming);
   if (e == cudaSuccess) bytes_ = block_bytes;
   return e;
 }
 
 namespace {
-// The calls below are allowed while a thread captures a stream (this one or
+// The calls below (a query, an allocation, user objects) are allowed while a thread captures a stream (this one or
 // another, in the global mode) only in the relaxed mode: otherwise they
 // invalidate its capture.
 struct RelaxedCapture {
@@ -88,12 +89,17 @@ void* SmallScratch::captured_block(unsigned long long capture, cudaStream_t stre
       const Captures::Slot& t = captures_->slot[k];
       if (t.taken && t.capture == capture && t.stream == stream) {
         captured_ = true;
-        return mem_ + (1 + k) * bytes_;
+        return captured_mem_[k];
       }
       if (!t.taken && free_slot == kCaptures) free_slot = k;
     }
     k = free_slot;
     if (k == kCaptures) return nullptr;
+    if (!captured_mem_[k] && cudaMalloc(&captured_mem_[k], bytes_) != cudaSuccess) {
+      cudaGetLastError();
+      captured_mem_[k] = nullptr;
+      return nullptr;
+    }
     captures_->slot[k].taken = true;
     captures_->slot[k].capture = capture;
     captures_->slot[k].stream = stream;
@@ -115,7 +121,7 @@ void* SmallScratch::captured_block(unsigned long long capture, cudaStream_t stre
     return nullptr;
   }
   captured_ = true;
-  return mem_ + (1 + k) * bytes_;
+  return captured_mem_[k];
 }
 
 }  // namespace fe

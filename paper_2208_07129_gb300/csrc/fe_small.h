@@ -15,8 +15,9 @@
 //  * captures: a captured product may run again at any time, so every pair of
 //    (capture, stream) has a block of its own, held until the graph and all
 //    that was instantiated from it are destroyed (a user object of the graph
-//    gives it back); kCaptures of them exist, later captures take the
-//    colour-ordered launches.
+//    gives it back).  The blocks are allocated when captures first ask for
+//    them, kCaptures at most, and kept for later captures; past these, or
+//    without memory, captured products take the colour-ordered launches.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -39,10 +40,11 @@ class SmallScratch {
   cudaError_t enqueued(cudaStream_t s);
 
  private:
-  static constexpr int kCaptures = 3;
+  static constexpr int kCaptures = 16;
   struct Captures;
   void* captured_block(unsigned long long capture, cudaStream_t stream, cudaGraph_t graph);
-  char* mem_ = nullptr;
+  char* mem_ = nullptr;                 // outside captures
+  char* captured_mem_[kCaptures] = {};
   size_t bytes_ = 0;
   cudaEvent_t done_ = nullptr;          // after the last product outside captures
   bool used_ = false, captured_ = false;

@@ -143,16 +143,16 @@ def test_more_captures_than_blocks(case, mode):
     their blocks back."""
     c = case(SMALL, False, mode)
     for _ in range(3):
-        Y = [torch.full_like(c.X[k & 1], float("nan")) for k in range(6)]
-        graphs = [c.capture(k & 1, Y[k]) for k in range(6)]
-        streams = [torch.cuda.Stream() for _ in range(6)]
+        Y = [torch.full_like(c.X[k & 1], float("nan")) for k in range(19)]
+        graphs = [c.capture(k & 1, Y[k]) for k in range(19)]
+        streams = [torch.cuda.Stream() for _ in range(19)]
         torch.cuda.synchronize()
         for _ in range(10):
             for g, s in zip(graphs, streams):
                 with torch.cuda.stream(s):
                     g.replay()
         torch.cuda.synchronize()
-        for k in range(6):
+        for k in range(19):
             assert torch.equal(Y[k], c.want[k & 1])
         del graphs
 
