@@ -226,6 +226,7 @@ struct fe_batch {
   size_t smem = 0;
   int grid = 0;
   std::vector<int> group_grid;         // persistent grid of each group's kernel
+  std::vector<size_t> group_smem;      // its shared memory: the largest tile of its own problems
   cudaStream_t cap = nullptr;
   std::vector<cudaStream_t> side;       // one capture branch per group
   cudaEvent_t fork = nullptr;
@@ -357,7 +358,8 @@ cudaError_t launch_group(fe_batch* b, int g, int n_g, size_t smem) {
 
 // Both steps for group g (degree p, n_q = p + 2).
 template <typename T>
-cudaError_t for_group(fe_batch* b, int g, size_t smem, bool launch) {
+cudaError_t for_group(fe_batch* b, int g, bool launch) {
+  const size_t smem = b->group_smem[g];
   const int n_g = b->item_begin[g + 1] - b->item_begin[g];
   switch (kind_of(b->ctxs[b->group_first[g]]->p)) {
     case 0: return launch ? launch_group<T, 4, 5>(b, g, n_g, smem) : prepare_group<T, 4, 5>(b, g, n_g, smem);
@@ -435,6 +437,8 @@ fe_status build_batch(fe_batch* b, int autotune_on) {
     }
     b->group_of[i] = g;
     if (!same_aspect(b->ctxs[b->group_first[g]], b->ctxs[i])) b->group_mixed[g] = 1;
+    b->group_smem.resize(b->group_first.size(), 0);
+    b->group_smem[g] = std::max(b->group_smem[g], tile_smem<T>(b->ctxs[i]->nq, b->vb[i]));
   }
   const int groups = (int)b->group_first.size();
   b->group_grid.assign(groups, 0);
@@ -518,7 +522,7 @@ fe_status build_batch(fe_batch* b, int autotune_on) {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     b->grid = std::max(1, std::min(b->n_items, std::max(1, per_sm) * sms));
   } else {
-    for (int g = 0; g < groups && e == cudaSuccess; ++g) e = for_group<T>(b, g, smem, false);
+    for (int g = 0; g < groups && e == cudaSuccess; ++g) e = for_group<T>(b, g, false);
   }
   if (e != cudaSuccess) return fe::cuda_status(e, where);
   where = "fe_batch_create: streams and events";
@@ -542,14 +546,16 @@ fe_status build_batch(fe_batch* b, int autotune_on) {
       e = cudaGetLastError();
       if (e != cudaSuccess) where = "fe_batch_create: captured resets of the queues";
     }
-    for (int g = 0; g < groups && e == cudaSuccess && !merged; ++g) {
-      e = cudaStreamWaitEvent(b->side[g], b->fork, 0);
-      if (e != cudaSuccess) { where = "fe_batch_create: fork of a group's branch"; break; }
-      e = for_group<T>(b, g, smem, true);
-      if (e != cudaSuccess) { where = "fe_batch_create: captured launch of a group's kernel"; break; }
-      e = cudaEventRecord(b->join[g], b->side[g]);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(b->cap, b->join[g], 0);
-      if (e != cudaSuccess) where = "fe_batch_create: join of a group's branch";
+    if constexpr (!merged) {
+      for (int g = 0; g < groups && e == cudaSuccess; ++g) {
+        e = cudaStreamWaitEvent(b->side[g], b->fork, 0);
+        if (e != cudaSuccess) { where = "fe_batch_create: fork of a group's branch"; break; }
+        e = for_group<T>(b, g, true);
+        if (e != cudaSuccess) { where = "fe_batch_create: captured launch of a group's kernel"; break; }
+        e = cudaEventRecord(b->join[g], b->side[g]);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(b->cap, b->join[g], 0);
+        if (e != cudaSuccess) where = "fe_batch_create: join of a group's branch";
+      }
     }
     cudaGraph_t g = nullptr;
     const cudaError_t e2 = cudaStreamEndCapture(b->cap, &g);
